@@ -137,7 +137,8 @@ typedef struct {
                             /* The cluster solver (exx_ctx_set_solver) ignores it.           */
     int precond;            /* EXX_PRECOND_MG (1, default of the Python binding): the mixed  */
                             /* path's CG is preconditioned by one multigrid V(1,1) cycle     */
-                            /* per iteration (weighted Jacobi smoothing, trilinear transfers, */
+                            /* per iteration on the second-order Laplacian of the same       */
+                            /* directions (weighted Jacobi smoothing, trilinear transfers,   */
                             /* Galerkin coarse operators built per plan on the host, the     */
                             /* inverse of the coarsest one), which cuts the iterations by    */
                             /* about a factor of ten.  The paper's CG is plain: only the     */
@@ -209,7 +210,9 @@ typedef struct {
  * exx_params at plan creation; chosen per plan by exx_plan_autotune. */
 typedef struct {
     int precond;            /* EXX_PRECOND_NONE or EXX_PRECOND_MG */
-    float omega;            /* weighted-Jacobi factor of the V-cycle, in (0, 1] (default 0.8) */
+    float omega;            /* weighted-Jacobi factor of the V-cycle, in (0, 1] (default 0.8), as */
+                            /* it would damp the CG's own stencil (the cycle's second-order one   */
+                            /* takes the factor that damps its highest frequency alike)           */
     int inner_shift;        /* reliable update (double-float true residual) once the FP32    */
                             /* residual fell by 2^-inner_shift, 4..22 (default 14)          */
     double ms;              /* exx_plan_autotune: measured solver time of the sample, ms    */

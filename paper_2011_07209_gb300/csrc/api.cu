@@ -250,13 +250,15 @@ static int upload_mg(exx_plan *p, int s, const SetLayout &L)
         return EXX_OK;
     }
     MgTables T;
-    int e = make_mg_tables(L, p->stencil, p->params.fd_order, kMgMinPoints, kMgOmega, kMgDrop, T);
+    if (!mg_definite(p->stencil)) return EXX_OK;
+    const double omega = kMgOmega * mg_omega_scale(p->params.fd_order);
+    int e = make_mg_tables(L, p->stencil, 1, kMgMinPoints, omega, kMgDrop, T);
     if (e) return e;
     if (T.nlev < 2) return EXX_OK;
     MgDev &G = p->h_mg[s];
     std::memset(&G, 0, sizeof(G));
     G.nlev = T.nlev;
-    G.omega = (float)kMgOmega;
+    G.omega = (float)omega;
     long long off = 0;
     for (int l = 1; l < T.nlev; ++l) {
         MgLevelDev &v = G.lv[l];
@@ -522,6 +524,7 @@ static void fill_celldev(const exx_plan *p, CellDev &C)
     fd_weights(n, w2, w1);
     for (int d = 0; d < st.ndir; ++d) {
         for (int k = 0; k < 3; ++k) C.dir[d][k] = st.dir[d][k];
+        C.coef[d] = (float)st.coef[d];
         for (int s = 0; s <= n; ++s) {
             C.cw64[d][s] = st.coef[d] * w2[s];
             C.cw32[d][s] = (float)C.cw64[d][s];
@@ -535,9 +538,9 @@ static void fill_celldev(const exx_plan *p, CellDev &C)
     C.r_pair2 = p->params.r_pair * p->params.r_pair;
     C.stress_mode = p->params.stress_mode;
     C.guess = p->params.guess;
-    C.precond = p->sched.precond;
+    C.precond = p->sched.precond && mg_definite(st);
     C.inner_shift = p->sched.inner_shift;
-    C.mg_omega = p->sched.omega;
+    C.mg_omega = (float)(p->sched.omega * mg_omega_scale(n));
     for (int s = 0; s < 2; ++s) {
         const SetLayout &L = p->lay[s];
         SetDev &S = C.set[s];

@@ -9,7 +9,7 @@ constexpr int kNlm = 49;   // (lmax + 1)^2 for lmax = 6; tables are padded to th
 
 // Multigrid preconditioner of the mixed-precision Step IV solve (V(1,1) cycle,
 // weighted Jacobi, trilinear transfers; not in the paper, whose CG is plain).
-// Level 0 is the set's dense CG box and its operator the kernel's stencil;
+// Level 0 is the set's dense CG box and its operator the second-order stencil (CellDev::coef);
 // coarse levels 1 .. nlev-2 are dense boxes with a margin of kMgPadDev points,
 // each row applied over a pattern of K offsets with the level's interior
 // weights (wrow = -1) or its own weights (a row of wexp); the coarsest level
@@ -35,7 +35,7 @@ struct MgLevelDev {
 };
 struct MgDev {
     int nlev;                      // levels including the fine one; 0: no hierarchy
-    float omega;                   // Jacobi weight (level 0 takes omega / diag of the stencil)
+    float omega;                   // Jacobi weight (level 0 takes omega / diag of its stencil)
     long long floats;              // floats of the slot region the coarse boxes need
     MgLevelDev lv[kMgLevelsDev];   // lv[1 .. nlev-1]
     int kd[kMgLevelsDev][kMgKDev]; // pattern offsets, (dx+2) | (dy+2) << 3 | (dz+2) << 6
@@ -104,6 +104,7 @@ struct CellDev {
     double cw64[6][8];             // coef_d * w2_s, s = 0..n
     float cw32[6][8];
     double w1dx[3][8];             // w1_s / dxi_alpha
+    float coef[6];                 // coef_d: the weight of the second-order stencil's neighbours
     double tol;
     int max_iter, precision;
     double r_pair2;
@@ -125,7 +126,7 @@ struct CellDev {
     int guess;                     // 1: CG starts from the free-space multipole potential
     int precond;                   // 1: multigrid-preconditioned mixed CG where the set has a hierarchy
     int inner_shift;               // reliable update after the FP32 residual fell by 2^-inner_shift (0: launch default)
-    float mg_omega;                // Jacobi weight of the V-cycle (0: the tables' own)
+    float mg_omega;                // Jacobi weight of the V-cycle's operator (0: the tables' own)
     // warm start: initial guesses from the previous solve of the same plan
     const int32_t *warm_map;       // [n_orb][n_orb] index of pair (i, j) in warm_rows, -1 none; NULL: cold
     const PairRec *warm_rows;

@@ -659,6 +659,8 @@ struct SmemCell {
     CellDev C;
     double cw64[6][8];
     float cw32[6][8];
+    float cwlo[6][8];    // the second-order stencil of the V-cycle, as cw32
+    float centerlo;
     float2 cwdf[6][8];   // cw64 as double-float pairs
     float2 centerdf;
     float cn[kNlm];      // N_l0 at l^2 + l, sqrt2 N_lm at l^2 + l + m (m > 0)
@@ -1240,13 +1242,16 @@ __device__ __forceinline__ void cg_mixed_sweep(const CgMixed &cg, int &iters, in
 // before and after the coarse correction, trilinear prolongation P and its
 // transpose as restriction, Galerkin operators P^T A P on the coarse levels
 // (built on the host per subdomain kind) and the inverse of the coarsest one.
-// On the fine level the Jacobi weight omega / diag(A) is one constant c0 (the
+// The cycle's own operator (A_2, L_2 = -A_2) is the second-order stencil of the same
+// directions, 7 to 13 points: as a preconditioner of the sixth-order A it costs no
+// iteration (13.0 either way on the 64-molecule cell) and a third of the reads.
+// On the fine level the Jacobi weight omega / diag(A_2) is one constant c0 (the
 // stencil's diagonal does not vary), so the pre-smoothed residual is
-// r - c0 A r and needs no stored pre-smoothed vector.
+// r - c0 A_2 r and needs no stored pre-smoothed vector.
 // ---------------------------------------------------------------------------
 struct MgSm {                      // the hierarchy of the pair's set, in shared memory
     int nlev;
-    float c0;                      // omega / diag(A) of the fine level
+    float c0;                      // omega / diag(A_2) of the fine level
     float dscale;                  // omega / (the tables' omega): scales the coarse dinv
     int n[kMgLevelsDev], K[kMgLevelsDev], Bp1[kMgLevelsDev], Bp2[kMgLevelsDev];
     int n_int[kMgLevelsDev], n_exp[kMgLevelsDev];
@@ -1646,7 +1651,8 @@ __device__ __forceinline__ void front_sweep(int ng, int nchunk, int W, const int
     }
 }
 
-__shared__ int g_mg_need[kMaxSweepChunks];   // update front of each chunk (multigrid path)
+// update front of each chunk (multigrid path): for the CG's stencil and, shorter, for the V-cycle's
+__shared__ int g_mg_need[kMaxSweepChunks], g_mg_need1[kMaxSweepChunks];
 
 struct MgScalars {
     double rz, rmax, S;
@@ -1661,25 +1667,23 @@ __shared__ MgScalars g_mg_cs;
 // the caller's frame across the call).  Each returns its thread's part of the
 // pass's dot product as a double-float pair (hi, lo).
 
-// t = r + c0 L r on one group (the stencil half of pass B and the frame's first
+// t = r + c0 L_2 r on one group (the stencil half of pass B and the frame's first
 // pre-smoothing), into qf
-template <int FDN>
 __device__ __forceinline__ void mg_pre_smooth_group(const SetDev &S, const SmemCell &sm, const float *__restrict__ rf,
                                                     float *__restrict__ qf, float c0, int g)
 {
     const int32_t gw = __ldg(S.groups + g);
     const int off = (gw >> 4) << 2, mask = gw & 15;
     float acc[4];
-    lap4<FDN>(rf, off, sm.cw32, sm.center32, S.rstride, S.d2, sm.C.ndir, acc);
+    lap4<1>(rf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.C.ndir, acc);
     const float4 r = ld4(rf + off);
     st4(qf + off, (mask & 1) ? r.x + c0 * acc[0] : 0.f, (mask & 2) ? r.y + c0 * acc[1] : 0.f,
         (mask & 4) ? r.z + c0 * acc[2] : 0.f, (mask & 8) ? r.w + c0 * acc[3] : 0.f);
 }
 
-template <int FDN>
 __device__ __noinline__ void mg_pre_smooth_all(const SetDev &S, const SmemCell &sm, const float *rf, float *qf, float c0)
 {
-    for (int g = threadIdx.x; g < S.n_groups; g += blockDim.x) mg_pre_smooth_group<FDN>(S, sm, rf, qf, c0, g);
+    for (int g = threadIdx.x; g < S.n_groups; g += blockDim.x) mg_pre_smooth_group(S, sm, rf, qf, c0, g);
 }
 
 // pass A: p = z + beta p (p = z in a frame's first iteration; z is in qf) ahead
@@ -1715,8 +1719,7 @@ __device__ __noinline__ float2 mg_pass_a(const SetDev &S, const SmemCell &sm, fl
     return make_float2(a.hi, a.lo);
 }
 
-// pass B: r -= alpha q, e += alpha p (<r, r>) ahead of t = r + c0 L r into qf
-template <int FDN>
+// pass B: r -= alpha q, e += alpha p (<r, r>) ahead of t = r + c0 L_2 r into qf
 __device__ __noinline__ float2 mg_pass_b(const SetDev &S, const SmemCell &sm, float *__restrict__ rf,
                                          float *__restrict__ qf, const float *__restrict__ pf, float *__restrict__ ef,
                                          float alpha, float c0, int nchunk, int W)
@@ -1724,7 +1727,7 @@ __device__ __noinline__ float2 mg_pass_b(const SetDev &S, const SmemCell &sm, fl
     const int32_t *__restrict__ grp = S.groups;
     DF b = {0.f, 0.f};
     front_sweep(
-        S.n_groups, nchunk, W, g_mg_need,
+        S.n_groups, nchunk, W, g_mg_need1,
         [&](int g) {
             const int off = (__ldg(grp + g) >> 4) << 2;
             const float4 r = ld4(rf + off), q = ld4(qf + off), p = ld4(pf + off), e = ld4(ef + off);
@@ -1733,15 +1736,14 @@ __device__ __noinline__ float2 mg_pass_b(const SetDev &S, const SmemCell &sm, fl
             st4(ef + off, e.x + alpha * p.x, e.y + alpha * p.y, e.z + alpha * p.z, e.w + alpha * p.w);
             df_add(b, r0 * r0 + r1 * r1 + r2 * r2 + r3 * r3);
         },
-        [&](int g) { mg_pre_smooth_group<FDN>(S, sm, rf, qf, c0, g); });
+        [&](int g) { mg_pre_smooth_group(S, sm, rf, qf, c0, g); });
     return make_float2(b.hi, b.lo);
 }
 
-// pass D: z0 = c0 r + P Z_1 into zf ahead of z = z0 + c0 (r + L z0) into qf, <r, z>.
+// pass D: z0 = c0 r + P Z_1 into zf ahead of z = z0 + c0 (r + L_2 z0) into qf, <r, z>.
 // The group's four points u2 .. u2+3 (u2 a multiple of 4) take their last-axis
 // parents from three level-1 values of each (x, y) row: one row, or two along
 // each axis whose fine coordinate is odd (pinfo).
-template <int FDN>
 __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, const float *__restrict__ rf,
                                          float *__restrict__ zf, float *__restrict__ qf, float c0, int nchunk, int W)
 {
@@ -1752,7 +1754,7 @@ __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, co
     const int cB2 = m.Bp2[1], sx = m.Bp1[1] * m.Bp2[1];
     DF a = {0.f, 0.f};
     front_sweep(
-        S.n_groups, nchunk, W, g_mg_need,
+        S.n_groups, nchunk, W, g_mg_need1,
         [&](int g) {
             const int32_t gw = __ldg(grp + g);
             const int off = (gw >> 4) << 2, mask = gw & 15;
@@ -1791,7 +1793,7 @@ __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, co
             const int32_t gw = __ldg(grp + g);
             const int off = (gw >> 4) << 2, mask = gw & 15;
             float acc[4];
-            const float4 z0 = lap4<FDN>(zf, off, sm.cw32, sm.center32, S.rstride, S.d2, sm.C.ndir, acc);
+            const float4 z0 = lap4<1>(zf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.C.ndir, acc);
             const float4 r = ld4(rf + off);
             const float z_0 = (mask & 1) ? z0.x + c0 * (r.x + acc[0]) : 0.f;
             const float z_1 = (mask & 2) ? z0.y + c0 * (r.y + acc[1]) : 0.f;
@@ -1808,9 +1810,9 @@ __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, co
 // region for the coarse boxes.  One PCG iteration is four passes over the fine
 // groups, each a pointwise update run ahead of a stencil (front_sweep):
 //   A  p = z + beta p           ahead of   q = A p, <p, q>
-//   B  r -= alpha q, e += alpha p   ahead of   t = r + c0 L r (pre-smoothed residual)
+//   B  r -= alpha q, e += alpha p   ahead of   t = r + c0 L_2 r (pre-smoothed residual)
 //      restriction of t, the coarse levels
-//   D  z0 = c0 r + P Z_1         ahead of   z = z0 + c0 (r + L z0), <r, z>
+//   D  z0 = c0 r + P Z_1         ahead of   z = z0 + c0 (r + L_2 z0), <r, z>
 // (pass B's t is discarded when its <r, r> calls for a reliable update).
 template <int FDN>
 __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mgbase, int &iters, int &refine,
@@ -1841,7 +1843,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
         if (tid == 0) {
             m.nlev = G.nlev;
             const double om = sm.C.mg_omega > 0.f ? (double)sm.C.mg_omega : (double)G.omega;
-            m.c0 = (float)(om / -(double)sm.center64);
+            m.c0 = (float)(om / -(double)sm.centerlo);
             m.dscale = (float)(om / (double)G.omega);
             m.cinv = G.cinv;
             m.pinfo = G.pinfo;
@@ -1889,9 +1891,9 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
     const int W = kSweepChunkGroups * nt;
     const int nchunk = (ng + W - 1) / W;
     {
-        int reach = 7;
-        for (int d = 0; d < ndir; ++d) reach = max(reach, 3 + FDN * max(abs(dsf[d]), abs(rs[d])));
-        for (int c = tid; c < nchunk; c += nt) {
+        int step = 0;   // longest stencil step
+        for (int d = 0; d < ndir; ++d) step = max(step, max(abs(dsf[d]), abs(rs[d])));
+        auto front = [&](int c, int reach) {
             const int last = min(ng, (c + 1) * W) - 1;
             const long long lim = (long long)((grp[last] >> 4) << 2) + reach;
             int lo = last + 1, hi = ng;
@@ -1900,7 +1902,11 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
                 if ((long long)((grp[mid] >> 4) << 2) <= lim) lo = mid + 1;
                 else hi = mid;
             }
-            g_mg_need[c] = lo;
+            return lo;
+        };
+        for (int c = tid; c < nchunk; c += nt) {
+            g_mg_need[c] = front(c, max(7, 3 + FDN * step));
+            g_mg_need1[c] = front(c, max(7, 3 + step));
         }
     }
     __syncthreads();
@@ -1914,7 +1920,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
         else mg_restrict(m, 0, qf, B1, B2, 0);
         __syncthreads();
         mg_coarse_cycle();
-        const float2 d = mg_pass_d<FDN>(S, sm, rf, zf, qf, c0, nchunk, W);
+        const float2 d = mg_pass_d(S, sm, rf, zf, qf, c0, nchunk, W);
         DF a[1] = {{d.x, d.y}};
         block_sum_df<1>(a, red2);
         return (double)a[0].hi + (double)a[0].lo;
@@ -1939,7 +1945,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
             __syncthreads();
         }
         // z = M r from the frame's residual (pass B without its update)
-        mg_pre_smooth_all<FDN>(S, sm, rf, qf, c0);
+        mg_pre_smooth_all(S, sm, rf, qf, c0);
         const double rz0 = finish_precondition();
         if (tid == 0) {
             cs.rz = rz0;
@@ -1972,7 +1978,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
             int act = cs.act;
             if (!act) {
                 // pass B: e += alpha p, r -= alpha q (<r, r>) ahead of t = r + c0 L r
-                const float2 pb = mg_pass_b<FDN>(S, sm, rf, qf, pf, ef, alpha, c0, nchunk, W);
+                const float2 pb = mg_pass_b(S, sm, rf, qf, pf, ef, alpha, c0, nchunk, W);
                 DF b[1] = {{pb.x, pb.y}};
                 block_sum_df<1>(b, red2);
                 if (tid == 0) {
@@ -2454,6 +2460,7 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
                 sm.cw64[d][s] = sm.C.cw64[d][s];
                 sm.cw32[d][s] = sm.C.cw32[d][s];
                 sm.cwdf[d][s] = dw_split(sm.C.cw64[d][s]);
+                sm.cwlo[d][s] = s == 1 ? sm.C.coef[d] : 0.f;
             } else if (tid >= 64 && tid < 64 + kNlm) {
                 const int lm = tid - 64;
                 int l = 0;
@@ -2480,6 +2487,9 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
                 sm.center64 = c;
                 sm.center32 = (float)c;
                 sm.centerdf = dw_split(c);
+                double lo = 0.0;
+                for (int d = 0; d < sm.C.ndir; ++d) lo -= 2.0 * (double)sm.C.coef[d];
+                sm.centerlo = (float)lo;
                 s_cell = pr.cell;
             }
             __syncthreads();

@@ -760,6 +760,22 @@ int make_mg_levels(const SetLayout &L, const Stencil &st, int fd_n, int min_poin
     return EXX_OK;
 }
 
+bool mg_definite(const Stencil &st)
+{
+    bool positive = true;   // every direction's coefficient: a sum of squares
+    for (int d = 0; d < st.ndir; ++d) positive &= st.coef[d] > 0.0;
+    return positive || negative_definite(st, 1);
+}
+
+double mg_omega_scale(int fd_n)
+{
+    double w2[kMaxFd + 1], w1[kMaxFd + 1];
+    fd_weights(fd_n, w2, w1);
+    double top = w2[0];   // the symbol at the highest frequency of a line
+    for (int s = 1; s <= fd_n; ++s) top += 2.0 * w2[s] * (s & 1 ? -1.0 : 1.0);
+    return top / w2[0] / 2.0;   // second order: 2
+}
+
 // Device form of the hierarchy (see plan.h).
 int make_mg_tables(const SetLayout &L, const Stencil &st, int fd_n, int min_points, double omega, double drop,
                    MgTables &t)

@@ -160,6 +160,19 @@ struct MgTables {
     std::vector<int32_t> pinfo1;
     long long slot_floats = 0;                      // three boxes per coarse level
 };
+// The V-cycle works on the second-order operator of the CG's directions (fd_n = 1 in
+// make_mg_tables) whatever the order of the CG's own stencil: its 7 to 13 points
+// cost the smoothing passes a third of the reads of the sixth-order stencil's 19 to
+// 37, and it is spectrally close enough that the CG takes as many iterations
+// (13.0 with either on the 64-molecule cell).
+// mg_definite: that operator is positive definite.  Always true so far wherever the CG's
+// own is (3000 random cells with a negative coefficient, shears to 1.3); the CG
+// is plain otherwise.
+bool mg_definite(const Stencil &st);
+// Jacobi factors are meant for the CG's operator: mg_omega_scale(fd_n) x omega is the
+// factor of the second-order one that damps its highest frequency alike (the ratio of
+// the largest eigenvalues of D^-1 A on a line: 1, 1.067 and 1.110 for fd_n = 1, 2, 3).
+double mg_omega_scale(int fd_n);
 // drop: pattern entries below drop x the interior diagonal are left out of the
 // device operators of the coarse levels (each added, as |a|, to its row's diagonal)
 int make_mg_tables(const SetLayout &L, const Stencil &st, int fd_n, int min_points, double omega, double drop,
