@@ -105,7 +105,8 @@ typedef struct {
     int lmax;               /* multipole order, 0..6 */
     int cg_max_iter;        /* cap on CG iterations per pair (summed over refinements) */
     int nq;                 /* NK candidate count N_q of Algorithm 1 (paper default 15) */
-    int precision;          /* EXX_FP64: every step in FP64.  EXX_MIXED: FP32 stencil and */
+    int precision;          /* EXX_FP64: every step in FP64 (see precond).  EXX_MIXED: FP32   */
+                            /* stencil and                                                */
                             /* axpy inside a true-residual refinement loop; dot products  */
                             /* exact-product double-float; moments and far field from     */
                             /* FP32 tables with FP64 sums; the true residuals, the        */
@@ -135,8 +136,8 @@ typedef struct {
                             /* quarter of the iterations; 0: from v = 0.  Only the starting  */
                             /* point changes: the stopping rule and the solution do not.     */
                             /* The cluster solver (exx_ctx_set_solver) ignores it.           */
-    int precond;            /* EXX_PRECOND_MG (1, default of the Python binding): the mixed  */
-                            /* path's CG is preconditioned by one multigrid V(1,1) cycle     */
+    int precond;            /* EXX_PRECOND_MG (1, default of the Python binding): the        */
+                            /* CG is preconditioned by one multigrid V(1,1) cycle            */
                             /* per iteration on the second-order Laplacian of the same       */
                             /* directions (weighted Jacobi smoothing, trilinear transfers,   */
                             /* Galerkin coarse operators built per plan on the host, the     */
@@ -144,8 +145,10 @@ typedef struct {
                             /* about a factor of ten.  The paper's CG is plain: only the     */
                             /* iterates change, not the discrete equations or the stopping   */
                             /* rule.  Used for fd_order <= 3 on the CTA solver; elsewhere,   */
-                            /* and with EXX_PRECOND_NONE (0), the CG is plain.  The FP64     */
-                            /* path is always plain CG.                                      */
+                            /* and with EXX_PRECOND_NONE (0), the CG is plain.  The cycle    */
+                            /* works in FP32; on the FP64 path it only proposes the search   */
+                            /* directions of a CG whose vectors, products, solution and      */
+                            /* residuals are FP64.                                           */
 } exx_params;
 
 typedef struct {
@@ -295,7 +298,7 @@ int exx_plan_set_schedule(exx_plan *plan, const exx_schedule *sched);
  * timing the solver launch with CUDA events on `stream`, twice per candidate
  * (the faster run counts), and keeps the fastest for the plan's later solves
  * (ties keep the earlier candidate, the order above).  `chosen` (may be NULL)
- * receives it with its time.  The FP64 path has one schedule (plain FP64 CG)
+ * receives it with its time.  The FP64 path has one schedule (of its parameters)
  * and returns it untimed.  A sample of several waves of the persistent grid
  * (a few times `ctas` of exx_plan_query) gives stable choices: with one wave
  * the slowest single pair decides each time.  cell and orb as for

@@ -233,13 +233,12 @@ static int mg_put(exx_plan *p, int s, const std::vector<T> &v, const T **out)
 }
 
 // The multigrid hierarchy of set s for the plan's current layout and stencil
-// (mixed precision with params.precond only; none when the set is too small
+// (with params.precond only; none when the set is too small
 // or the stencil reaches too far for the coarse boxes).
 static int upload_mg(exx_plan *p, int s, const SetLayout &L)
 {
     free_mg(p, s);
-    if (p->params.precision != EXX_MIXED || p->params.precond != EXX_PRECOND_MG || p->params.fd_order > 3)
-        return EXX_OK;
+    if (p->params.precond != EXX_PRECOND_MG || p->params.fd_order > 3) return EXX_OK;
     if (s == 1 && p->off[1].m == p->off[0].m) {
         // the same offset set (equal self and non-self radii): the same hierarchy
         if (p->d_mg[0]) {
@@ -538,7 +537,8 @@ static void fill_celldev(const exx_plan *p, CellDev &C)
     C.r_pair2 = p->params.r_pair * p->params.r_pair;
     C.stress_mode = p->params.stress_mode;
     C.guess = p->params.guess;
-    C.precond = p->sched.precond && mg_definite(st);
+    // the FP64 path takes its preconditioner from the parameters: schedules are the mixed path's
+    C.precond = (p->params.precision == EXX_MIXED ? p->sched.precond : p->params.precond) && mg_definite(st);
     C.inner_shift = p->sched.inner_shift;
     C.mg_omega = (float)(p->sched.omega * mg_omega_scale(n));
     for (int s = 0; s < 2; ++s) {
@@ -811,8 +811,9 @@ int exx_plan_create(exx_ctx *ctx, const exx_cell *cell, const exx_params *params
     p->sched.omega = (float)kMgOmega;
     p->sched.inner_shift = ctx->inner_shift;
     e = build_geometry(p);
-    if (!e && p->sched.precond == EXX_PRECOND_MG && !p->d_mg[0] && !p->d_mg[1])
-        p->sched.precond = EXX_PRECOND_NONE;   // no hierarchy for this plan: plain CG
+    if (!e && p->sched.precond == EXX_PRECOND_MG &&
+        (params->precision != EXX_MIXED || (!p->d_mg[0] && !p->d_mg[1])))
+        p->sched.precond = EXX_PRECOND_NONE;   // no hierarchy for this plan (plain CG), or no schedule (FP64)
     if (!e) {
         const long long pairs = (long long)max_orb * (max_orb + 1) / 2;
         p->pairs_cap = (int)std::min<long long>(pairs, 1LL << 30);
@@ -1411,7 +1412,9 @@ int exx_plan_set_schedule(exx_plan *plan, const exx_schedule *sched)
     if (sched->precond != EXX_PRECOND_NONE && sched->precond != EXX_PRECOND_MG) return EXX_ERR_ARG;
     if (!(sched->omega > 0.f && sched->omega <= 1.f) || sched->inner_shift < 4 || sched->inner_shift > 22)
         return EXX_ERR_ARG;
-    if (sched->precond == EXX_PRECOND_MG && !plan->d_mg[0] && !plan->d_mg[1]) return EXX_ERR_ARG;
+    if (sched->precond == EXX_PRECOND_MG &&
+        (plan->params.precision != EXX_MIXED || (!plan->d_mg[0] && !plan->d_mg[1])))
+        return EXX_ERR_ARG;
     plan->sched = *sched;
     return EXX_OK;
 }

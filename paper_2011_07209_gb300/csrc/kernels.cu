@@ -1805,39 +1805,15 @@ __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, co
     return make_float2(a.hi, a.lo);
 }
 
-// The mixed-precision solve of one pair with the multigrid preconditioner (see
-// the comment above MgSm).  zf: one more dense FP32 box; mgbase: the slot's
-// region for the coarse boxes.  One PCG iteration is four passes over the fine
-// groups, each a pointwise update run ahead of a stencil (front_sweep):
-//   A  p = z + beta p           ahead of   q = A p, <p, q>
-//   B  r -= alpha q, e += alpha p   ahead of   t = r + c0 L_2 r (pre-smoothed residual)
-//      restriction of t, the coarse levels
-//   D  z0 = c0 r + P Z_1         ahead of   z = z0 + c0 (r + L_2 z0), <r, z>
-// (pass B's t is discarded when its <r, r> calls for a reliable update).
-template <int FDN>
-__device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mgbase, int &iters, int &refine,
-                                         int &status, double &rnorm, double *es, bool &es_done)
+// The hierarchy of the pair's set into shared memory, its coarse boxes (mgbase) zeroed,
+// and the update fronts of the fused passes (stencil half-width fdn); nchunk chunks of W groups.
+__device__ __noinline__ void mg_setup(const SetDev &S, const SmemCell &sm, float *mgbase, int fdn, int &nchunk, int &W)
 {
-    es_done = false;
-    const SetDev &S = *cg.S;
-    const SmemCell &sm = *cg.sm;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    float *__restrict__ pf = cg.pf;
-    float *__restrict__ rf = cg.rf;
-    float *__restrict__ qf = cg.qf;
-    float *__restrict__ ef = cg.ef;
-    float2 *vb = reinterpret_cast<float2 *>(cg.vbox);
-    float *r32 = reinterpret_cast<float *>(cg.r64);
-    const int32_t *__restrict__ poff = S.pe_off;
-    const int32_t *__restrict__ grp = S.groups;
-    const int npe = S.n_pe, ng = S.n_groups, ndir = cg.ndir;
-    const int *rs = S.rstride, *dsf = S.dstride;
-    const double stop = cg.stop, inner_red = cg.inner_red;
-    float2 *red2 = reinterpret_cast<float2 *>(cg.red);
-    const int B1 = S.B[1], B2 = S.B[2];
-
     MgSm &m = g_mg_sm;
-    MgScalars &cs = g_mg_cs;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int32_t *__restrict__ grp = S.groups;
+    const int *rs = S.rstride, *dsf = S.dstride;
+    const int ng = S.n_groups, ndir = sm.C.ndir;
     {
         const MgDev &G = *S.mg;
         if (tid == 0) {
@@ -1888,13 +1864,14 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
         for (long long k = tid; k < G.floats; k += nt) mgbase[k] = 0.f;
     }
     // update front of every chunk of the fused passes
-    const int W = kSweepChunkGroups * nt;
-    const int nchunk = (ng + W - 1) / W;
+    W = kSweepChunkGroups * nt;
+    nchunk = (ng + W - 1) / W;
+    const int w = W;
     {
         int step = 0;   // longest stencil step
         for (int d = 0; d < ndir; ++d) step = max(step, max(abs(dsf[d]), abs(rs[d])));
         auto front = [&](int c, int reach) {
-            const int last = min(ng, (c + 1) * W) - 1;
+            const int last = min(ng, (c + 1) * w) - 1;
             const long long lim = (long long)((grp[last] >> 4) << 2) + reach;
             int lo = last + 1, hi = ng;
             while (lo < hi) {
@@ -1905,11 +1882,48 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
             return lo;
         };
         for (int c = tid; c < nchunk; c += nt) {
-            g_mg_need[c] = front(c, max(7, 3 + FDN * step));
+            g_mg_need[c] = front(c, max(7, 3 + fdn * step));
             g_mg_need1[c] = front(c, max(7, 3 + step));
         }
     }
     __syncthreads();
+}
+
+// The mixed-precision solve of one pair with the multigrid preconditioner (see
+// the comment above MgSm).  zf: one more dense FP32 box; mgbase: the slot's
+// region for the coarse boxes.  One PCG iteration is four passes over the fine
+// groups, each a pointwise update run ahead of a stencil (front_sweep):
+//   A  p = z + beta p           ahead of   q = A p, <p, q>
+//   B  r -= alpha q, e += alpha p   ahead of   t = r + c0 L_2 r (pre-smoothed residual)
+//      restriction of t, the coarse levels
+//   D  z0 = c0 r + P Z_1         ahead of   z = z0 + c0 (r + L_2 z0), <r, z>
+// (pass B's t is discarded when its <r, r> calls for a reliable update).
+template <int FDN>
+__device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mgbase, int &iters, int &refine,
+                                         int &status, double &rnorm, double *es, bool &es_done)
+{
+    es_done = false;
+    const SetDev &S = *cg.S;
+    const SmemCell &sm = *cg.sm;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    float *__restrict__ pf = cg.pf;
+    float *__restrict__ rf = cg.rf;
+    float *__restrict__ qf = cg.qf;
+    float *__restrict__ ef = cg.ef;
+    float2 *vb = reinterpret_cast<float2 *>(cg.vbox);
+    float *r32 = reinterpret_cast<float *>(cg.r64);
+    const int32_t *__restrict__ poff = S.pe_off;
+    const int32_t *__restrict__ grp = S.groups;
+    const int npe = S.n_pe, ng = S.n_groups, ndir = cg.ndir;
+    const int *rs = S.rstride, *dsf = S.dstride;
+    const double stop = cg.stop, inner_red = cg.inner_red;
+    float2 *red2 = reinterpret_cast<float2 *>(cg.red);
+    const int B1 = S.B[1], B2 = S.B[2];
+
+    MgSm &m = g_mg_sm;
+    MgScalars &cs = g_mg_cs;
+    int nchunk, W;
+    mg_setup(S, sm, mgbase, FDN, nchunk, W);
     if (!(cg.r0n > stop)) return;   // the starting guess already meets the tolerance
     const float c0 = m.c0;
 
@@ -2029,6 +2043,98 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
             __syncthreads();
         }
     }
+}
+
+// The FP64 solve of one pair with the same preconditioner: the CG's vectors, products
+// and residuals stay in FP64 (x in vbox, r in r64, p in pd, q in qd); the V-cycle only
+// proposes directions, z = M r, for which it takes r scaled to norm one in FP32 (rf; t and z
+// in tf, z0 in zf).  The line search alpha = <p, r> / <p, q> and the conjugation
+// beta = -<z, q> / <p, q> are formed in FP64 from the vectors themselves, so nothing rests
+// on M being applied exactly.  FP64 runs at 1/64 of the FP32 rate: an iteration of plain CG
+// costs about four V-cycles, and the CG takes a tenth of the iterations.
+__device__ __noinline__ void cg_fp64_mg(const SetDev &S, const SmemCell &sm, double *vbox, const double *rho, double *r64,
+                                        double *pd, double *qd, float *rf, float *tf, float *zf, float *mgbase,
+                                        double stop, double rr, double *red, int &iters, int &refine, int &status,
+                                        double &rnorm)
+{
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int ndir = sm.C.ndir, fdn = sm.C.fd_n, npe = S.n_pe;
+    const int32_t *__restrict__ poff = S.pe_off;
+    int nchunk, W;
+    mg_setup(S, sm, mgbase, fdn, nchunk, W);
+    const MgSm &m = g_mg_sm;
+    bool first = true;   // no previous direction
+    double pq_old = 0.0;
+    for (;;) {
+        // ended at a fifth of the bound: its error is then no larger than plain CG's, whose last
+        // iterations take smaller steps (one iteration more)
+        if (sqrt(rr) <= 0.2 * stop) {
+            rr = residual_pass(S, vbox, rho, r64, sm.cw64, sm.ds, ndir, fdn, sm.center64, red);
+            ++refine;
+            if (sqrt(rr) <= stop) break;
+            first = true;
+        }
+        if (iters >= sm.C.max_iter || !(rr == rr)) {
+            status = 5;
+            break;
+        }
+        // z = M r
+        const double sc = 1.0 / sqrt(rr);
+        for (int k = tid; k < npe; k += nt) rf[poff[k]] = (float)(r64[k] * sc);
+        __syncthreads();
+        mg_pre_smooth_all(S, sm, rf, tf, m.c0);
+        __syncthreads();
+        if (m.n_groups[1] > 0) mg_restrict_runs(tf, S.B[1], S.B[2]);
+        else mg_restrict(m, 0, tf, S.B[1], S.B[2], 0);
+        __syncthreads();
+        mg_coarse_cycle();
+        mg_pass_d(S, sm, rf, zf, tf, m.c0, nchunk, W);
+        __syncthreads();
+        double beta = 0.0;
+        if (!first) {
+            double zq[1] = {0.0};
+            for (int k = tid; k < npe; k += nt) zq[0] += (double)tf[poff[k]] * qd[k];
+            block_sum<1>(zq, red);
+            beta = -zq[0] / pq_old;
+        }
+        for (int k = tid; k < npe; k += nt) {
+            const int off = poff[k];
+            pd[off] = first ? (double)tf[off] : (double)tf[off] + beta * pd[off];
+        }
+        __syncthreads();
+        double dots[2] = {0.0, 0.0};   // <p, q>, <p, r>
+        for (int k = tid; k < npe; k += nt) {
+            const int off = poff[k];
+            const double q = -lap_at<double>(pd, off, sm.cw64, sm.ds, ndir, fdn, sm.center64), p = pd[off];
+            qd[k] = q;
+            dots[0] += p * q;
+            dots[1] += p * r64[k];
+        }
+        block_sum<2>(dots, red);
+        ++iters;
+        if (!(dots[0] > 0.0) || !(dots[1] > 0.0)) {   // a broken recurrence: start again from r, at most once
+            if (first) {
+                status = 5;
+                break;
+            }
+            first = true;
+            continue;
+        }
+        first = false;
+        pq_old = dots[0];
+        const double alpha = dots[1] / dots[0];
+        double rn[1] = {0.0};
+        for (int k = tid; k < npe; k += nt) {
+            const int off = poff[k];
+            vbox[off] += alpha * pd[off];
+            const double r = r64[k] - alpha * qd[k];
+            r64[k] = r;
+            rn[0] += r * r;
+        }
+        block_sum<1>(rn, red);
+        rr = rn[0];
+    }
+    rnorm = sqrt(rr);
 }
 
 // Starting guess of the CG: the free-space potential of rho on the PE points,
@@ -2509,6 +2615,8 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
         // double-float arithmetic; the others keep FP64 throughout
         const bool dfm = mixed && fdn <= 4 &&
                          (S.n_groups + kSweepChunkGroups * nt - 1) / (kSweepChunkGroups * nt) <= kMaxSweepChunks;
+        const bool mg64 = !mixed && C.precond && S.mg && fdn <= 3 &&
+                          (S.n_groups + kSweepChunkGroups * nt - 1) / (kSweepChunkGroups * nt) <= kMaxSweepChunks;
         float2 *vb = reinterpret_cast<float2 *>(vbox);
         float2 *b2 = reinterpret_cast<float2 *>(slot + W.off_b2);
         float *r32 = reinterpret_cast<float *>(r64);
@@ -2688,11 +2796,15 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
         }
         double es[10];   // Step V sums of the double-float path (valid in thread 0)
         if (!mixed) {
-            // plain FP64 CG: x in vbox (PE), r in r64, p in pbox, q in qv
+            // FP64 CG, plain or preconditioned: x in vbox (PE), r in r64, p in pbox, q in qv
             double *pd = (double *)pbox;
             double *qd = (double *)qv;
             double rr = rr2;
-            if (bn > 0.0) {
+            if (bn > 0.0 && mg64) {
+                cg_fp64_mg(S, sm, vbox, rho, r64, pd, qd, reinterpret_cast<float *>(rv), reinterpret_cast<float *>(ev),
+                           reinterpret_cast<float *>(slot + W.off_zf), reinterpret_cast<float *>(slot + W.off_mg), stop, rr,
+                           red, iters, refine, status, rnorm);
+            } else if (bn > 0.0) {
                 for (int k = tid; k < S.n_pe; k += nt) pd[S.pe_off[k]] = r64[k];
                 __syncthreads();
                 for (;;) {
@@ -2857,6 +2969,11 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
                 reinterpret_cast<float *>(slot + W.off_zf)[off] = 0.f;
             } else {
                 ((double *)qv)[k] = 0.0;   // q of the FP64 CG (compressed); the other paths read this region as a box
+                if (mg64) {   // its FP32 boxes (cg_fp64_mg)
+                    ((float *)rv)[off] = 0.f;
+                    ((float *)ev)[off] = 0.f;
+                    reinterpret_cast<float *>(slot + W.off_zf)[off] = 0.f;
+                }
             }
         }
         for (int h = tid; h < S.n_halo; h += nt) vbox[S.halo_off[h]] = 0.0;
