@@ -2,7 +2,7 @@
 //
 //   k_tables       regular solid harmonics on PE points and far-field kernels
 //                  on shell points of one subdomain kind (Eqs. me, mepole)
-//   k_pair_rows    unique pair list, one CTA per orbital row (Step II)
+//   k_pair_rows    unique pair list, a few orbital rows per CTA (Step II)
 //   k_pair_scan    row offsets and per-cell ranges of the pair list
 //   k_pair_solve   persistent: one CTA owns one pair at a time and runs the
 //                  whole per-pair path (Steps III-V): pair density, moments,
@@ -127,57 +127,39 @@ __global__ void k_tables(const CellDev *__restrict__ cell, int which, double *S6
 }
 
 // ---------------------------------------------------------------------------
-// Pair list: the rule of pair_rule.cuh, one CTA per orbital row.
+// Pair list: the rule of pair_rule.cuh.
 // ---------------------------------------------------------------------------
-// One CTA of kRowThreads per orbital row (cell, i).  fill = 0: count; 1: write.
-__global__ void __launch_bounds__(kRowThreads) k_pair_rows(const CellDev *__restrict__ cells, int n_cells,
-                                                          ListDev L, int fill)
+// kPairRows rows of one cell per CTA.  fill = 0: count; 1: write.
+__global__ void __launch_bounds__(kPairThreads) k_pair_rows(const CellDev *__restrict__ cells, int n_cells, ListDev L,
+                                                           int fill)
 {
-    const int row = blockIdx.x;
-    int c = 0;
-    while (c + 1 < n_cells && row >= cells[c + 1].row_base) ++c;
-    const CellDev &C = cells[c];
-    const int i = row - C.row_base;
-    if (i >= C.n_orb) return;
-    __shared__ int warp_tot[kRowThreads / 32];
-    __shared__ int s_base;
-    if (threadIdx.x == 0) s_base = fill ? L.row_start[row] : 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int j0 = i; j0 < C.n_orb; j0 += kRowThreads) {
-        const int j = j0 + threadIdx.x;
-        int kb[3], g[3];
-        const bool ok = (j < C.n_orb) && pair_rule(C, i, j, kb, g);
-        const unsigned bal = __ballot_sync(0xffffffffu, ok);
-        if (lane == 0) warp_tot[w] = __popc(bal);
-        __syncthreads();
-        int before = 0, tot = 0;
-        for (int k = 0; k < kRowThreads / 32; ++k) {
-            if (k < w) before += warp_tot[k];
-            tot += warp_tot[k];
-        }
-        if (fill && ok) {
-            const int pos = s_base + before + __popc(bal & ((1u << lane) - 1u));
-            if (pos < L.capacity) {
-                PairRec pr;
-                pr.i = i;
-                pr.j = j;
-                pr.k[0] = kb[0];
-                pr.k[1] = kb[1];
-                pr.k[2] = kb[2];
-                pr.g[0] = g[0];
-                pr.g[1] = g[1];
-                pr.g[2] = g[2];
-                pr.cell = c;
-                pr.pad = 0;
-                L.pairs[pos] = pr;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_base += tot;
-        __syncthreads();
+    int c = 0, b = blockIdx.x;
+    for (; c < n_cells; ++c) {
+        const int nb = (cells[c].n_orb + kPairRows - 1) / kPairRows;
+        if (b < nb) break;
+        b -= nb;
     }
-    if (!fill && threadIdx.x == 0) L.row_count[row] = s_base;
+    if (c == n_cells) return;
+    const CellDev &C = cells[c];
+    const int i0 = b * kPairRows, row0 = C.row_base + i0;
+    int cnt[kPairRows];
+    pair_rows_block(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
+        if (!fill) return;
+        const int pos = L.row_start[row0 + r] + p;
+        if (pos >= L.capacity) return;
+        PairRec pr;
+        pr.i = i0 + r;
+        pr.j = j;
+        for (int a = 0; a < 3; ++a) {
+            pr.k[a] = kb[a];
+            pr.g[a] = g[a];
+        }
+        pr.cell = c;
+        pr.pad = 0;
+        L.pairs[pos] = pr;
+    });
+    if (!fill && threadIdx.x == 0)
+        for (int r = 0; r < kPairRows && i0 + r < C.n_orb; ++r) L.row_count[row0 + r] = cnt[r];
 }
 
 // Exclusive scan of the row counts (single CTA), per-cell ranges, capacity check.
@@ -3846,9 +3828,10 @@ cudaError_t launch_guess_info(const int32_t *perm, const uint8_t *bin, const int
 
 cudaError_t launch_pair_list(const CellDev *cells, int n_cells, int n_rows, const ListDev &L, cudaStream_t s)
 {
-    if (n_rows > 0) k_pair_rows<<<n_rows, kRowThreads, 0, s>>>(cells, n_cells, L, 0);
+    const int blocks = n_rows / kPairRows + n_cells;   // a cell's last rows may fill a CTA only in part
+    if (n_rows > 0) k_pair_rows<<<blocks, kPairThreads, 0, s>>>(cells, n_cells, L, 0);
     k_pair_scan<<<1, 1024, 0, s>>>(cells, n_cells, n_rows, L);
-    if (n_rows > 0) k_pair_rows<<<n_rows, kRowThreads, 0, s>>>(cells, n_cells, L, 1);
+    if (n_rows > 0) k_pair_rows<<<blocks, kPairThreads, 0, s>>>(cells, n_cells, L, 1);
     return cudaGetLastError();
 }
 

@@ -6,7 +6,6 @@
 
 namespace exx {
 
-constexpr int kRowThreads = 128;     // pair-list CTA size
 // two 512-thread CTAs per SM, each on its own pair: one CTA's barriers and
 // per-pair passes overlap the other's streaming passes (64 registers a thread
 // either way)

@@ -24,7 +24,6 @@
 namespace {
 
 constexpr int kMaxOrbNoalloc = 16384;          // rows the static scratch can hold
-constexpr int kThreads = 128;
 
 // [0, kMax) pair count of each row, [kMax, 2 kMax) first pair of each row,
 // [2 kMax] total number of pairs.
@@ -38,46 +37,25 @@ struct PairCell {
     int n_orb;
 };
 
-// One CTA per row i; fill = 0 counts, fill = 1 writes rows in (i, j) order.
-__global__ void __launch_bounds__(kThreads) k_rows_noalloc(PairCell C, int *scratch, int fill, int cap, int *rows)
+// kPairRows rows per CTA; fill = 0 counts, fill = 1 writes rows in (i, j) order.
+__global__ void __launch_bounds__(exx::kPairThreads) k_rows_noalloc(PairCell C, int *scratch, int fill, int cap, int *rows)
 {
-    const int i = blockIdx.x;
-    __shared__ int warp_tot[kThreads / 32];
-    __shared__ int s_base;
-    if (threadIdx.x == 0) s_base = fill ? scratch[kMaxOrbNoalloc + i] : 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int j0 = i; j0 < C.n_orb; j0 += kThreads) {
-        const int j = j0 + threadIdx.x;
-        int kb[3], g[3];
-        const bool ok = (j < C.n_orb) && exx::pair_rule(C, i, j, kb, g);
-        const unsigned bal = __ballot_sync(0xffffffffu, ok);
-        if (lane == 0) warp_tot[w] = __popc(bal);
-        __syncthreads();
-        int before = 0, tot = 0;
-        for (int k = 0; k < kThreads / 32; ++k) {
-            if (k < w) before += warp_tot[k];
-            tot += warp_tot[k];
+    const int i0 = blockIdx.x * exx::kPairRows;
+    int cnt[exx::kPairRows];
+    exx::pair_rows_block(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
+        if (!fill) return;
+        const int pos = scratch[kMaxOrbNoalloc + i0 + r] + p;
+        if (pos >= cap) return;
+        int *o = rows + 8 * (size_t)pos;
+        o[0] = i0 + r;
+        o[1] = j;
+        for (int a = 0; a < 3; ++a) {
+            o[2 + a] = kb[a];
+            o[5 + a] = g[a];
         }
-        if (fill && ok) {
-            const int pos = s_base + before + __popc(bal & ((1u << lane) - 1u));
-            if (pos < cap) {
-                int *r = rows + 8 * (size_t)pos;
-                r[0] = i;
-                r[1] = j;
-                r[2] = kb[0];
-                r[3] = kb[1];
-                r[4] = kb[2];
-                r[5] = g[0];
-                r[6] = g[1];
-                r[7] = g[2];
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_base += tot;
-        __syncthreads();
-    }
-    if (!fill && threadIdx.x == 0) scratch[i] = s_base;
+    });
+    if (!fill && threadIdx.x == 0)
+        for (int r = 0; r < exx::kPairRows && i0 + r < C.n_orb; ++r) scratch[i0 + r] = cnt[r];
 }
 
 // Exclusive scan of the row counts (one CTA); writes the total to the scratch
@@ -202,9 +180,10 @@ extern "C" int exx_pair_list_noalloc(const exx_cell *cell, const double *centres
     C.n_orb = n_orb;
     cudaStream_t s = (cudaStream_t)stream;
     // the counts of every row are rewritten below; nothing else needs zeroing
-    if (n_orb > 0) k_rows_noalloc<<<n_orb, kThreads, 0, s>>>(C, scratch, 0, cap, rows);
+    const int blocks = (n_orb + exx::kPairRows - 1) / exx::kPairRows;
+    if (n_orb > 0) k_rows_noalloc<<<blocks, exx::kPairThreads, 0, s>>>(C, scratch, 0, cap, rows);
     k_scan_noalloc<<<1, 1024, 0, s>>>(scratch, n_orb, n_pairs);
-    if (n_orb > 0) k_rows_noalloc<<<n_orb, kThreads, 0, s>>>(C, scratch, 1, cap, rows);
+    if (n_orb > 0) k_rows_noalloc<<<blocks, exx::kPairThreads, 0, s>>>(C, scratch, 1, cap, rows);
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return exx::note_cuda_error("noalloc.cu: launch", ce);
     return EXX_OK;
