@@ -437,7 +437,8 @@ static bool same_directions(const Stencil &a, const Stencil &b)
 // cell, as Algorithm 1 runs at the beginning of every MD step (Sec. III C);
 // frozen = 2: the plan cell's aux directions are kept as well.  When the
 // directions change, the dense layouts are rebuilt from the same offsets (the
-// halo check runs again there).
+// halo check runs again there); otherwise they stand: layout and halo depend on the
+// offsets, the directions and the half-width alone.
 static int update_metric(exx_plan *p, const exx_cell &cell)
 {
     Metric m;
@@ -451,14 +452,6 @@ static int update_metric(exx_plan *p, const exx_cell &cell)
         e = make_stencil(m, p->params.fd_order, p->params.nq, nullptr, 0, st);
     if (e) return e;
     const bool relayout = !same_directions(st, p->stencil);
-    if (!relayout) {
-        // same directions: the layout stands; re-check the halo for safety
-        for (int s = 0; s < 2; ++s) {
-            SetLayout L;
-            e = make_layout(p->off[s], st, p->params.fd_order, L);
-            if (e) return e;
-        }
-    }
     p->metric = m;
     p->stencil = st;
     p->cell = cell;
@@ -472,26 +465,43 @@ static int update_metric(exx_plan *p, const exx_cell &cell)
 static int upload_guess_bins(exx_plan *p)
 {
     const double rpe[2] = {p->params.r_pe_self, p->params.r_pe_pair};
+    std::vector<uint8_t> bin;
+    std::vector<int32_t> count, perm;
     for (int s = 0; s < 2; ++s) {
         const OffsetSet &o = p->off[s];
         const int n = o.n_pe;
         if (n == 0 || !p->d_gs_perm[s]) continue;
-        std::vector<uint8_t> bin(n);
-        std::vector<int32_t> count(kGuessBins + 1, 0), perm(n);
-        for (int k = 0; k < n; ++k) {
-            double r2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-                double x = 0.0;
-                for (int al = 0; al < 3; ++al) x += p->metric.h[a][al] * o.m[3 * k + al] / p->metric.n[al];
-                r2 += x * x;
+        if (s == 0 || rpe[1] != rpe[0] || p->off[1].m != p->off[0].m) {   // equal sets have equal bins
+            bin.assign(n, 0);
+            count.assign(kGuessBins + 1, 0);
+            perm.resize(n);
+            // h m / N of each lattice axis, once per coordinate instead of once per point
+            int lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+            for (int k = 0; k < n; ++k)
+                for (int al = 0; al < 3; ++al) {
+                    lo[al] = std::min(lo[al], o.m[3 * k + al]);
+                    hi[al] = std::max(hi[al], o.m[3 * k + al]);
+                }
+            std::vector<double> step[3];
+            for (int al = 0; al < 3; ++al)
+                for (int m = lo[al]; m <= hi[al]; ++m)
+                    for (int a = 0; a < 3; ++a) step[al].push_back(p->metric.h[a][al] * m / p->metric.n[al]);
+            for (int k = 0; k < n; ++k) {
+                const double *t[3];
+                for (int al = 0; al < 3; ++al) t[al] = &step[al][(size_t)3 * (o.m[3 * k + al] - lo[al])];
+                double r2 = 0.0;
+                for (int a = 0; a < 3; ++a) {
+                    const double x = t[0][a] + t[1][a] + t[2][a];
+                    r2 += x * x;
+                }
+                const int b = (int)std::min<double>(kGuessBins - 1, std::sqrt(r2) / rpe[s] * kGuessBins);
+                bin[k] = (uint8_t)std::max(0, b);
+                count[bin[k] + 1]++;
             }
-            const int b = (int)std::min<double>(kGuessBins - 1, std::sqrt(r2) / rpe[s] * kGuessBins);
-            bin[k] = (uint8_t)std::max(0, b);
-            count[bin[k] + 1]++;
+            for (int b = 0; b < kGuessBins; ++b) count[b + 1] += count[b];
+            std::vector<int32_t> fill(count.begin(), count.end() - 1);
+            for (int k = 0; k < n; ++k) perm[fill[bin[k]]++] = k;
         }
-        for (int b = 0; b < kGuessBins; ++b) count[b + 1] += count[b];
-        std::vector<int32_t> fill(count.begin(), count.end() - 1);
-        for (int k = 0; k < n; ++k) perm[fill[bin[k]]++] = k;
         CK(cudaMemcpy(p->d_gs_perm[s], perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(p->d_gs_bstart[s], count.data(), 4 * (size_t)(kGuessBins + 1), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(p->d_gs_bin[s], bin.data(), (size_t)n, cudaMemcpyHostToDevice));

@@ -267,6 +267,12 @@ int choose_aux(const Metric &mt, const std::vector<Cand> &cands, int aux[3][3])
 // Symbol of the operator at wave vector t: sum_dir coef (w0 + 2 sum_q w_q cos(q t.d)).
 bool negative_definite(const Stencil &st, int n)
 {
+    // Central second differences of any order have a symbol below zero at every frequency but
+    // zero, so positive coefficients along three independent axes settle it (almost every
+    // cell does); the scan over frequencies took 9 ms of an MD step's 35 ms on the host.
+    bool positive = true;
+    for (int d = 0; d < st.ndir; ++d) positive &= st.coef[d] > 0.0;
+    if (positive) return true;
     double w2[kMaxFd + 1], w1[kMaxFd + 1];
     fd_weights(n, w2, w1);
     const int G = 32;
@@ -760,12 +766,7 @@ int make_mg_levels(const SetLayout &L, const Stencil &st, int fd_n, int min_poin
     return EXX_OK;
 }
 
-bool mg_definite(const Stencil &st)
-{
-    bool positive = true;   // every direction's coefficient: a sum of squares
-    for (int d = 0; d < st.ndir; ++d) positive &= st.coef[d] > 0.0;
-    return positive || negative_definite(st, 1);
-}
+bool mg_definite(const Stencil &st) { return negative_definite(st, 1); }
 
 double mg_omega_scale(int fd_n)
 {
