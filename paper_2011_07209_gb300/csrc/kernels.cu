@@ -2633,44 +2633,37 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
 
         // ---- multipole moments Q_lm = dV sum_PE rho r^l Y_lm (Eq. mepole) ----
         float *gs = reinterpret_cast<float *>(slot + W.off_gs);
-        if (mixed && S.gs_perm) {
+        if (mixed) {
             // by radial bin: the same pass gives the moments of the starting guess
             bin_moments(S, C, rho, gs, qpart);
         } else {
+            // The PE set is its own mirror image (|h m / N| <= R_PE holds for -m with m; in
+            // lexicographic order the mirror of point k is n_pe - 1 - k) and
+            // r^l Y_lm(-r) = (-1)^l r^l Y_lm(r): one half of the points, with
+            // rho(r) + rho(-r) for even l and the difference for odd l, in half the FP64 products
             double a0 = 0.0, a1 = 0.0;
-            const int nchunk = (S.n_pe + 31) >> 5;
-            // 32 points per step (rows past the end repeat the last one with weight 0),
+            const int half = (S.n_pe + 1) / 2, nchunk = (half + 31) >> 5;
+            // 32 rows per step (rows past the end repeat the last one with weight 0),
             // unrolled so that the table rows of several points are in flight at once
             const int lane1 = lane + 32 < kNlm ? lane + 32 : lane;
-            const float sel1 = lane + 32 < kNlm ? 1.f : 0.f;
+            const double sel1 = lane + 32 < kNlm ? 1.0 : 0.0;
+            auto odd = [](int lm) { return lm >= 25 ? lm < 36 : lm >= 9 ? lm < 16 : lm >= 1 && lm < 4; };   // l = 1, 3, 5
+            const bool o0 = odd(lane), o1 = odd(lane1);
             for (int ch = warp; ch < nchunk; ch += nwarps) {
-                const int k0 = ch << 5;
-                const double rl = (k0 + lane < S.n_pe) ? rho[k0 + lane] : 0.0;
-                const int last = min(32, S.n_pe - k0) - 1;
-                if (mixed) {
-                    float f0 = 0.f, f1 = 0.f;
-                    const float rlf = (float)rl;
-#pragma unroll 8
-                    for (int p = 0; p < 32; ++p) {
-                        const float rp = __shfl_sync(0xffffffffu, rlf, p);
-                        const float *row = S.S32 + (size_t)(k0 + min(p, last)) * kNlm;
-                        f0 += rp * row[lane];
-                        f1 += rp * row[lane1];
-                    }
-                    a0 += f0;
-                    a1 += sel1 * f1;
-                } else {
-                    double f0 = 0.0, f1 = 0.0;
+                const int k0 = ch << 5, k = k0 + lane, mir = S.n_pe - 1 - k;
+                const double ra = k < half ? rho[k] : 0.0, rb = k < half && mir != k ? rho[mir] : 0.0;
+                const double re = ra + rb, ro = ra - rb;
+                const int last = min(32, half - k0) - 1;
+                double f0 = 0.0, f1 = 0.0;
 #pragma unroll 4
-                    for (int p = 0; p < 32; ++p) {
-                        const double rp = __shfl_sync(0xffffffffu, rl, p);
-                        const double *row = S.S64 + (size_t)(k0 + min(p, last)) * kNlm;
-                        f0 += rp * row[lane];
-                        f1 += rp * row[lane1];
-                    }
-                    a0 += f0;
-                    a1 += sel1 * f1;
+                for (int p = 0; p < 32; ++p) {
+                    const double pe = __shfl_sync(0xffffffffu, re, p), po = __shfl_sync(0xffffffffu, ro, p);
+                    const double *row = S.S64 + (size_t)(k0 + min(p, last)) * kNlm;
+                    f0 += (o0 ? po : pe) * row[lane];
+                    f1 += (o1 ? po : pe) * row[lane1];
                 }
+                a0 += f0;
+                a1 += sel1 * f1;
             }
             qpart[warp][lane] = a0;
             if (lane + 32 < kNlm) qpart[warp][lane + 32] = a1;
