@@ -655,6 +655,7 @@ struct SmemCell {
     double center64;
     float center32;
     int ds[6];
+    int pair[2];         // direction (1,0,+-1), (0,1,+-1) whose rows axis 0, 1 reads too; -1: none (lap4)
 };
 
 // The mixed-precision Poisson solve of one pair (see the comment inside).
@@ -884,11 +885,16 @@ __device__ __forceinline__ void st4s(float *p, float a, float b, float c, float 
 // boundary at the s_-th neighbour: the two aligned groups around that point
 // hold all four values, picked by compile-time indices (the sign of d2[d] is
 // the same for every thread).  Each group read holds at least one of the
-// values needed, so no read leaves the box.  Longer steps along the contiguous
-// axis read point by point.
-template <int FDN>
+// values needed, so no read leaves the box.  The directions (1,0,+-1) and (0,1,+-1)
+// meet the rows that the axes 0 and 1 read anyway (pair[0], pair[1]): with SHARE their
+// aligned groups are read once, 33 float4 instead of 45 for the 37-point stencil of a
+// triclinic cell and 13 instead of 17 for the second-order one, whose reads bound the
+// passes (L1 wavefronts).  SHARE is for stencils that have such directions: the
+// groups' longer life costs the 64 registers more than nothing (19 points: pass A 3.6 -> 4.1
+// ms a pair).  Longer steps along the contiguous axis read point by point.
+template <int FDN, bool SHARE>
 __device__ __forceinline__ float4 lap4(const float *__restrict__ x_, int off, const float (*cw)[8], float center,
-                                       const int *rs, const int *d2, int ndir, float (&acc)[4])
+                                       const int *rs, const int *d2, const int *pair, int ndir, float (&acc)[4])
 {
     const float4 c = ld4(x_ + off);
     const float4 cm = ld4(x_ + off - 4);
@@ -900,41 +906,45 @@ __device__ __forceinline__ float4 lap4(const float *__restrict__ x_, int off, co
     for (int s_ = 1; s_ <= FDN; ++s_)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] += cw[2][s_] * (x[4 + i + s_] + x[4 + i - s_]);
+    // a direction with a last-axis step of +-1: f(off + i + s_ ds) = f(bp + i + s_ d2) and
+    // f(off + i - s_ ds) = f(bm + i - s_ d2) with bp, bm = off +- s_ rs on group boundaries;
+    // p, m: the groups at bp and bm, already read
+    auto slant = [&](int s_, float w, bool up, int bp, int bm, const float4 &p, const float4 &m) {
+        if (up) {
+            const float4 p1 = ld4(x_ + bp + 4), m0 = ld4(x_ + bm - 4);   // bp .. bp+7, bm-4 .. bm+3
+            const float P[8] = {p.x, p.y, p.z, p.w, p1.x, p1.y, p1.z, p1.w};
+            const float M[8] = {m0.x, m0.y, m0.z, m0.w, m.x, m.y, m.z, m.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += w * (P[i + s_] + M[4 + i - s_]);
+        } else {
+            const float4 p0 = ld4(x_ + bp - 4), m1 = ld4(x_ + bm + 4);   // bp-4 .. bp+3, bm .. bm+7
+            const float P[8] = {p0.x, p0.y, p0.z, p0.w, p.x, p.y, p.z, p.w};
+            const float M[8] = {m.x, m.y, m.z, m.w, m1.x, m1.y, m1.z, m1.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += w * (P[4 + i - s_] + M[i + s_]);
+        }
+    };
 #pragma unroll
     for (int d = 0; d < 6; ++d) {
-        if (d == 2 || d >= ndir) continue;
+        if (d == 2 || d >= ndir || (SHARE && d > 2 && (d == pair[0] || d == pair[1]))) continue;
         if (d2[d] == 0) {
+            // pair[d]: the slanted direction that meets axis d's rows takes their groups along
+            const int e = SHARE && d < 2 ? pair[d] : -1;
 #pragma unroll
             for (int s_ = 1; s_ <= FDN; ++s_) {
-                const float4 a = ld4(x_ + off + s_ * rs[d]);
-                const float4 b = ld4(x_ + off - s_ * rs[d]);
+                const int bp = off + s_ * rs[d], bm = off - s_ * rs[d];
+                const float4 a = ld4(x_ + bp), b = ld4(x_ + bm);
                 acc[0] += cw[d][s_] * (a.x + b.x);
                 acc[1] += cw[d][s_] * (a.y + b.y);
                 acc[2] += cw[d][s_] * (a.z + b.z);
                 acc[3] += cw[d][s_] * (a.w + b.w);
+                if (e >= 0) slant(s_, cw[e][s_], d2[e] > 0, bp, bm, a, b);
             }
         } else if (d2[d] == 1 || d2[d] == -1) {
-            // f(off + i + s_ dsf) = f(bp + i + s_ d2) and f(off + i - s_ dsf) = f(bm + i - s_ d2)
-            // with bp, bm = off +- s_ rs[d] on group boundaries
-            const bool up = d2[d] > 0;
 #pragma unroll
             for (int s_ = 1; s_ <= FDN; ++s_) {
                 const int bp = off + s_ * rs[d], bm = off - s_ * rs[d];
-                if (up) {
-                    const float4 p0 = ld4(x_ + bp), p1 = ld4(x_ + bp + 4);   // bp .. bp+7
-                    const float4 m0 = ld4(x_ + bm - 4), m1 = ld4(x_ + bm);   // bm-4 .. bm+3
-                    const float P[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-                    const float M[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[i] += cw[d][s_] * (P[i + s_] + M[4 + i - s_]);
-                } else {
-                    const float4 p0 = ld4(x_ + bp - 4), p1 = ld4(x_ + bp);   // bp-4 .. bp+3
-                    const float4 m0 = ld4(x_ + bm), m1 = ld4(x_ + bm + 4);   // bm .. bm+7
-                    const float P[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-                    const float M[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[i] += cw[d][s_] * (P[4 + i - s_] + M[i + s_]);
-                }
+                slant(s_, cw[d][s_], d2[d] > 0, bp, bm, ld4(x_ + bp), ld4(x_ + bm));
             }
         } else {
             // longer steps along the contiguous axis (auxiliary directions beyond the first shell)
@@ -954,13 +964,13 @@ __device__ __forceinline__ float4 lap4(const float *__restrict__ x_, int off, co
 template <int FDN>
 __device__ __forceinline__ void stencil_group(const float *__restrict__ pf, const float *__restrict__ rf,
                                               float *__restrict__ qf, int32_t gw, const float (*cw)[8], float center,
-                                              const int *rs, const int *dsf, const int *d2, int ndir, DF &apq, DF &aqq,
+                                              const int *rs, const int *d2, const int *pair, int ndir, DF &apq, DF &aqq,
                                               DF &arq, DF &arp)
 {
     const int off = (gw >> 4) << 2;
     const int mask = gw & 15;
     float acc[4];
-    const float4 c = lap4<FDN>(pf, off, cw, center, rs, d2, ndir, acc);
+    const float4 c = lap4<FDN, false>(pf, off, cw, center, rs, d2, pair, ndir, acc);
     const float q0 = (mask & 1) ? -acc[0] : 0.f, q1 = (mask & 2) ? -acc[1] : 0.f;
     const float q2 = (mask & 4) ? -acc[2] : 0.f, q3 = (mask & 8) ? -acc[3] : 0.f;
     st4s(qf + off, q0, q1, q2, q3);
@@ -1159,7 +1169,7 @@ __device__ __forceinline__ void cg_mixed_sweep(const CgMixed &cg, int &iters, in
         DF dv[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};   // <p,q> <q,q> <r,q> <r,p> <r,r>
         if (!pending) {
             for (int g = tid; g < ng; g += nt)
-                stencil_group<FDN>(pf, rf, qf, __ldg(grp + g), cw, center, rs, dsf, d2, ndir, dv[0], dv[1], dv[2],
+                stencil_group<FDN>(pf, rf, qf, __ldg(grp + g), cw, center, rs, d2, sm.pair, ndir, dv[0], dv[1], dv[2],
                                    dv[3]);
         } else {
             int front = 0;
@@ -1172,7 +1182,7 @@ __device__ __forceinline__ void cg_mixed_sweep(const CgMixed &cg, int &iters, in
                 __syncthreads();
                 const int gend = min(ng, (c + 1) * W);
                 for (int g = c * W + tid; g < gend; g += nt)
-                    stencil_group<FDN>(pf, rf, qf, __ldg(grp + g), cw, center, rs, dsf, d2, ndir, dv[0], dv[1], dv[2],
+                    stencil_group<FDN>(pf, rf, qf, __ldg(grp + g), cw, center, rs, d2, sm.pair, ndir, dv[0], dv[1], dv[2],
                                        dv[3]);
             }
         }
@@ -1252,15 +1262,6 @@ struct MgSm {                      // the hierarchy of the pair's set, in shared
     int nrow1, rows1[25];          // level 1: (dx, dy) rows of the window with pattern entries
     float cr[kMgCoarsestDev];
 };
-
-// L x on the four lanes of one aligned group (the stencil of stencil_group).
-template <int FDN>
-__device__ __forceinline__ void lap_group(const float *__restrict__ x_, int off, const float (*cw)[8], float center,
-                                          const int *rs, const int *dsf, const int *d2, int ndir, float (&acc)[4])
-{
-    (void)dsf;
-    lap4<FDN>(x_, off, cw, center, rs, d2, ndir, acc);
-}
 
 __device__ __forceinline__ void mg_coords(int o, int B1, int B2, int &u0, int &u1, int &u2)
 {
@@ -1657,7 +1658,7 @@ __device__ __forceinline__ void mg_pre_smooth_group(const SetDev &S, const SmemC
     const int32_t gw = __ldg(S.groups + g);
     const int off = (gw >> 4) << 2, mask = gw & 15;
     float acc[4];
-    lap4<1>(rf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.C.ndir, acc);
+    lap4<1, true>(rf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.pair, sm.C.ndir, acc);
     const float4 r = ld4(rf + off);
     st4(qf + off, (mask & 1) ? r.x + c0 * acc[0] : 0.f, (mask & 2) ? r.y + c0 * acc[1] : 0.f,
         (mask & 4) ? r.z + c0 * acc[2] : 0.f, (mask & 8) ? r.w + c0 * acc[3] : 0.f);
@@ -1670,7 +1671,7 @@ __device__ __noinline__ void mg_pre_smooth_all(const SetDev &S, const SmemCell &
 
 // pass A: p = z + beta p (p = z in a frame's first iteration; z is in qf) ahead
 // of q = A p into qf, <p, q>
-template <int FDN>
+template <int FDN, bool SHARE>
 __device__ __noinline__ float2 mg_pass_a(const SetDev &S, const SmemCell &sm, float *__restrict__ pf,
                                          float *__restrict__ qf, float beta, bool copy, int nchunk, int W)
 {
@@ -1692,7 +1693,7 @@ __device__ __noinline__ float2 mg_pass_a(const SetDev &S, const SmemCell &sm, fl
             const int32_t gw = __ldg(grp + g);
             const int off = (gw >> 4) << 2, mask = gw & 15;
             float acc[4];
-            const float4 p = lap4<FDN>(pf, off, sm.cw32, sm.center32, S.rstride, S.d2, sm.C.ndir, acc);
+            const float4 p = lap4<FDN, SHARE>(pf, off, sm.cw32, sm.center32, S.rstride, S.d2, sm.pair, sm.C.ndir, acc);
             const float q0 = (mask & 1) ? -acc[0] : 0.f, q1 = (mask & 2) ? -acc[1] : 0.f;
             const float q2 = (mask & 4) ? -acc[2] : 0.f, q3 = (mask & 8) ? -acc[3] : 0.f;
             st4(qf + off, q0, q1, q2, q3);
@@ -1775,7 +1776,7 @@ __device__ __noinline__ float2 mg_pass_d(const SetDev &S, const SmemCell &sm, co
             const int32_t gw = __ldg(grp + g);
             const int off = (gw >> 4) << 2, mask = gw & 15;
             float acc[4];
-            const float4 z0 = lap4<1>(zf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.C.ndir, acc);
+            const float4 z0 = lap4<1, true>(zf, off, sm.cwlo, sm.centerlo, S.rstride, S.d2, sm.pair, sm.C.ndir, acc);
             const float4 r = ld4(rf + off);
             const float z_0 = (mask & 1) ? z0.x + c0 * (r.x + acc[0]) : 0.f;
             const float z_1 = (mask & 2) ? z0.y + c0 * (r.y + acc[1]) : 0.f;
@@ -1908,6 +1909,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
     mg_setup(S, sm, mgbase, FDN, nchunk, W);
     if (!(cg.r0n > stop)) return;   // the starting guess already meets the tolerance
     const float c0 = m.c0;
+    const bool share = sm.pair[0] >= 0 || sm.pair[1] >= 0;   // lap4
 
     // restriction, coarse levels and pass D: z into qf, <r, z> returned (valid in warp 0)
     auto finish_precondition = [&]() -> double {
@@ -1960,7 +1962,8 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
             const float beta = cs.beta;
             const bool copy = first;
             first = false;
-            const float2 pa = mg_pass_a<FDN>(S, sm, pf, qf, beta, copy, nchunk, W);
+            const float2 pa = share ? mg_pass_a<FDN, true>(S, sm, pf, qf, beta, copy, nchunk, W)
+                                    : mg_pass_a<FDN, false>(S, sm, pf, qf, beta, copy, nchunk, W);
             DF a[1] = {{pa.x, pa.y}};
             block_sum_df<1>(a, red2);
             if (tid == 0) {
@@ -2576,6 +2579,11 @@ __global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) k_pair_solve(c
             if (tid == 0) {
                 double c = 0.0;
                 for (int d = 0; d < sm.C.ndir; ++d) c += sm.C.cw64[d][0];
+                sm.pair[0] = sm.pair[1] = -1;
+                for (int d = 3; d < sm.C.ndir; ++d) {
+                    const int *v = sm.C.dir[d];
+                    if ((v[2] == 1 || v[2] == -1) && v[0] + v[1] == 1 && v[0] * v[1] == 0) sm.pair[v[0] == 1 ? 0 : 1] = d;
+                }
                 sm.center64 = c;
                 sm.center32 = (float)c;
                 sm.centerdf = dw_split(c);
