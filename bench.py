@@ -577,7 +577,7 @@ def run_trajectory(args, rank, world, local_rank):
         del dxx, runs
         torch.cuda.empty_cache()
 
-    # plain FP64 GPU path beside the mixed one on a pair sample of MD step 0 (the
+    # FP64 GPU path (its CG preconditioned as the mixed one's) beside it on a pair sample of MD step 0 (the
     # pairs of its first --arm-orbitals MLWFs), and both against the FP64 oracle
     arms, accuracy, cpu = None, None, None
     if rank == 0 and not args.no_arms and not shard:

@@ -2035,8 +2035,9 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
 // proposes directions, z = M r, for which it takes r scaled to norm one in FP32 (rf; t and z
 // in tf, z0 in zf).  The line search alpha = <p, r> / <p, q> and the conjugation
 // beta = -<z, q> / <p, q> are formed in FP64 from the vectors themselves, so nothing rests
-// on M being applied exactly.  FP64 runs at 1/64 of the FP32 rate: an iteration of plain CG
-// costs about four V-cycles, and the CG takes a tenth of the iterations.
+// on M being applied exactly.  Bound by the FP64 stencil (37 points, N_PE = 118k, one CTA
+// on an SM: 5.8 ms an iteration, about ten V-cycles), of which the CG now takes a tenth: the
+// first 32 orbitals of the 128-molecule triclinic cell 904 -> 108 ms.
 __device__ __noinline__ void cg_fp64_mg(const SetDev &S, const SmemCell &sm, double *vbox, const double *rho, double *r64,
                                         double *pd, double *qd, float *rf, float *tf, float *zf, float *mgbase,
                                         double stop, double rr, double *red, int &iters, int &refine, int &status,
