@@ -119,6 +119,9 @@ struct exx_plan {
     double *d_S64[2] = {}, *d_T64[2] = {};
     float *d_S32[2] = {}, *d_T32[2] = {};
     bool tables_valid = false;
+    // metric, stencil, offsets, layouts and their device tables belong together and to `cell`;
+    // false after an upload that failed part way: the next solve builds all of it again
+    bool geometry_valid = false;
     // device copies for host-memory inputs
     int max_orb = 0;
     int box[3] = {};
@@ -331,16 +334,24 @@ static void free_geometry(exx_plan *p)
     p->warm_n = 0;   // the offsets change: stored solutions no longer apply
 }
 
-// Offsets, stencil and layout for cell0 (and the aux directions to freeze).
-// Dense CG layouts of both offset sets for the plan's current stencil (box
-// margins, strides, groups and halo order depend on the stencil directions),
-// uploaded to the device.
-static int upload_layouts(exx_plan *p)
+// Dense CG layouts of both offset sets for a stencil (box margins, strides, groups
+// and halo order depend on its directions); the halo check is made here.
+static int make_layouts(const OffsetSet (&off)[2], const Stencil &st, int fd_order, SetLayout (&lay)[2])
 {
     for (int s = 0; s < 2; ++s) {
-        SetLayout L;
-        int e = make_layout(p->off[s], p->stencil, p->params.fd_order, L);
+        const int e = make_layout(off[s], st, fd_order, lay[s]);
         if (e) return e;
+    }
+    return EXX_OK;
+}
+
+// The layouts (of the plan's current offsets and stencil) become the plan's and are
+// uploaded to the device.
+static int upload_layouts(exx_plan *p, SetLayout (&lay)[2])
+{
+    for (int s = 0; s < 2; ++s) {
+        SetLayout &L = lay[s];
+        int e;
         dev_free(p->d_pe_m[s]);
         dev_free(p->d_pe_off[s]);
         dev_free(p->d_sh_m[s]);
@@ -391,22 +402,35 @@ static int upload_layouts(exx_plan *p)
     return EXX_OK;
 }
 
-// Offsets, stencil and layout for cell0 (and the aux directions to freeze).
-static int build_geometry(exx_plan *p)
+// Offsets, stencil and layout for a cell (and the aux directions to freeze): all of it
+// on the host first, so that a cell that is refused leaves the plan as it was.
+static int build_geometry(exx_plan *p, const exx_cell &cell)
 {
-    int e = make_metric(p->cell0.lattice, p->cell0.n, p->metric);
+    Metric m;
+    Stencil st;
+    OffsetSet off[2];
+    SetLayout lay[2];
+    int e = make_metric(cell.lattice, cell.n, m);
     if (e) return e;
-    e = make_stencil(p->metric, p->params.fd_order, p->params.nq, nullptr, 0, p->stencil);
+    e = make_stencil(m, p->params.fd_order, p->params.nq, nullptr, 0, st);
     if (e) return e;
-    p->n_aux = p->stencil.n_aux;
-    for (int a = 0; a < 3; ++a)
-        for (int k = 0; k < 3; ++k) p->aux[a][k] = a < p->n_aux ? p->stencil.dir[3 + a][k] : 0;
     const double rpe[2] = {p->params.r_pe_self, p->params.r_pe_pair};
     const double rme[2] = {p->params.r_me_self, p->params.r_me_pair};
-    free_geometry(p);
     for (int s = 0; s < 2; ++s) {
-        e = make_offsets(p->metric, rpe[s], rme[s], p->off[s]);
+        e = make_offsets(m, rpe[s], rme[s], off[s]);
         if (e) return e;
+    }
+    if ((e = make_layouts(off, st, p->params.fd_order, lay))) return e;
+    p->geometry_valid = false;
+    free_geometry(p);
+    p->cell0 = p->cell = cell;
+    p->metric = m;
+    p->stencil = st;
+    p->n_aux = st.n_aux;
+    for (int a = 0; a < 3; ++a)
+        for (int k = 0; k < 3; ++k) p->aux[a][k] = a < p->n_aux ? st.dir[3 + a][k] : 0;
+    for (int s = 0; s < 2; ++s) {
+        p->off[s] = std::move(off[s]);
         const OffsetSet &o = p->off[s];
         if ((e = dev_alloc(&p->d_S64[s], (size_t)o.n_pe * kNlm)) ||
             (e = dev_alloc(&p->d_S32[s], (size_t)o.n_pe * kNlm)) ||
@@ -417,9 +441,8 @@ static int build_geometry(exx_plan *p)
             (e = dev_alloc(&p->d_gs_S32[s], (size_t)o.n_pe * kNlm)) || (e = dev_alloc(&p->d_gs_info[s], (size_t)o.n_pe)))
             return e;
     }
-    if ((e = upload_layouts(p))) return e;
-    p->cell = p->cell0;
-    p->tables_valid = false;
+    if ((e = upload_layouts(p, lay))) return e;
+    p->geometry_valid = true;
     return EXX_OK;
 }
 
@@ -438,7 +461,8 @@ static bool same_directions(const Stencil &a, const Stencil &b)
 // frozen = 2: the plan cell's aux directions are kept as well.  When the
 // directions change, the dense layouts are rebuilt from the same offsets (the
 // halo check runs again there); otherwise they stand: layout and halo depend on the
-// offsets, the directions and the half-width alone.
+// offsets, the directions and the half-width alone.  A cell that is refused leaves the
+// plan as it was, so that the next cell is checked against what the layouts belong to.
 static int update_metric(exx_plan *p, const exx_cell &cell)
 {
     Metric m;
@@ -452,11 +476,17 @@ static int update_metric(exx_plan *p, const exx_cell &cell)
         e = make_stencil(m, p->params.fd_order, p->params.nq, nullptr, 0, st);
     if (e) return e;
     const bool relayout = !same_directions(st, p->stencil);
+    SetLayout lay[2];
+    if (relayout && (e = make_layouts(p->off, st, p->params.fd_order, lay))) return e;
     p->metric = m;
     p->stencil = st;
     p->cell = cell;
     p->tables_valid = false;
-    if (relayout && (e = upload_layouts(p))) return e;
+    if (relayout) {
+        p->geometry_valid = false;
+        if ((e = upload_layouts(p, lay))) return e;
+        p->geometry_valid = true;
+    }
     return EXX_OK;
 }
 
@@ -813,14 +843,13 @@ int exx_plan_create(exx_ctx *ctx, const exx_cell *cell, const exx_params *params
     if (!p) return EXX_ERR_OOM;
     p->ctx = ctx;
     p->device = ctx->device;
-    p->cell0 = *cell;
     p->params = *params;
     p->max_orb = max_orb;
     for (int a = 0; a < 3; ++a) p->box[a] = box[a];
     p->sched.precond = params->precond;
     p->sched.omega = (float)kMgOmega;
     p->sched.inner_shift = ctx->inner_shift;
-    e = build_geometry(p);
+    e = build_geometry(p, *cell);
     if (!e && p->sched.precond == EXX_PRECOND_MG &&
         (params->precision != EXX_MIXED || (!p->d_mg[0] && !p->d_mg[1])))
         p->sched.precond = EXX_PRECOND_NONE;   // no hierarchy for this plan (plain CG), or no schedule (FP64)
@@ -1049,13 +1078,12 @@ int exx_pairs_solve_batch(exx_ctx *ctx, int n_cells, exx_plan *const *plans, con
     // geometry for the current cells
     for (int c = 0; c < n_cells; ++c) {
         exx_plan *p = plans[c];
-        if (same_cell(cells[c], p->cell)) continue;
-        int e;
+        int e = EXX_OK;
         if (p->params.frozen) {
-            e = update_metric(p, cells[c]);
-        } else {
-            p->cell0 = cells[c];
-            e = build_geometry(p);
+            if (!p->geometry_valid) e = build_geometry(p, p->cell0);
+            if (!e && !same_cell(cells[c], p->cell)) e = update_metric(p, cells[c]);
+        } else if (!p->geometry_valid || !same_cell(cells[c], p->cell)) {
+            e = build_geometry(p, cells[c]);
         }
         if (e) return e;
     }
