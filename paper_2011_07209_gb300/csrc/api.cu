@@ -109,6 +109,7 @@ struct exx_plan {
     exx_params params{};
     Metric metric{};
     Stencil stencil{};
+    bool mg_ok = false;    // the V-cycle's operator for this stencil is definite (v_cycle_definite)
     int aux[3][3] = {};
     int n_aux = 0;
     OffsetSet off[2];
@@ -235,13 +236,21 @@ static int mg_put(exx_plan *p, int s, const std::vector<T> &v, const T **out)
     return EXX_OK;
 }
 
+// Whether a plan's solves may use the V-cycle with this stencil.  Asked when the stencil is
+// set, not per solve: with a negative coefficient (strongly sheared cells) the answer takes a
+// scan over frequencies, 3 ms of host time, more than the whole solve of a small cell.
+static bool v_cycle_definite(const exx_params &P, const Stencil &st)
+{
+    return P.precond == EXX_PRECOND_MG && P.fd_order <= 3 && mg_definite(st);
+}
+
 // The multigrid hierarchy of set s for the plan's current layout and stencil
-// (with params.precond only; none when the set is too small
+// (with params.precond and a definite operator only; none when the set is too small
 // or the stencil reaches too far for the coarse boxes).
 static int upload_mg(exx_plan *p, int s, const SetLayout &L)
 {
     free_mg(p, s);
-    if (p->params.precond != EXX_PRECOND_MG || p->params.fd_order > 3) return EXX_OK;
+    if (!p->mg_ok) return EXX_OK;
     if (s == 1 && p->off[1].m == p->off[0].m) {
         // the same offset set (equal self and non-self radii): the same hierarchy
         if (p->d_mg[0]) {
@@ -252,7 +261,6 @@ static int upload_mg(exx_plan *p, int s, const SetLayout &L)
         return EXX_OK;
     }
     MgTables T;
-    if (!mg_definite(p->stencil)) return EXX_OK;
     const double omega = kMgOmega * mg_omega_scale(p->params.fd_order);
     int e = make_mg_tables(L, p->stencil, 1, kMgMinPoints, omega, kMgDrop, T);
     if (e) return e;
@@ -426,6 +434,7 @@ static int build_geometry(exx_plan *p, const exx_cell &cell)
     p->cell0 = p->cell = cell;
     p->metric = m;
     p->stencil = st;
+    p->mg_ok = v_cycle_definite(p->params, st);
     p->n_aux = st.n_aux;
     for (int a = 0; a < 3; ++a)
         for (int k = 0; k < 3; ++k) p->aux[a][k] = a < p->n_aux ? st.dir[3 + a][k] : 0;
@@ -480,6 +489,7 @@ static int update_metric(exx_plan *p, const exx_cell &cell)
     if (relayout && (e = make_layouts(p->off, st, p->params.fd_order, lay))) return e;
     p->metric = m;
     p->stencil = st;
+    p->mg_ok = v_cycle_definite(p->params, st);
     p->cell = cell;
     p->tables_valid = false;
     if (relayout) {
@@ -578,7 +588,7 @@ static void fill_celldev(const exx_plan *p, CellDev &C)
     C.stress_mode = p->params.stress_mode;
     C.guess = p->params.guess;
     // the FP64 path takes its preconditioner from the parameters: schedules are the mixed path's
-    C.precond = (p->params.precision == EXX_MIXED ? p->sched.precond : p->params.precond) && mg_definite(st);
+    C.precond = (p->params.precision == EXX_MIXED ? p->sched.precond : p->params.precond) && p->mg_ok;
     C.inner_shift = p->sched.inner_shift;
     C.mg_omega = (float)(p->sched.omega * mg_omega_scale(n));
     for (int s = 0; s < 2; ++s) {

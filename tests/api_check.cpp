@@ -6,6 +6,7 @@
 //   step <9 lattice>   solve one orbital in this cell: status, and whether the solver was launched on a
 //                      layout that is the one of the stencil it was given
 //   oom <k>            the k-th device allocation from now on fails (0: none)
+//   scans              how often mg_definite was asked since the last time
 //   layout <9 lattice> <3 n> <9 lattice> r_pe r_me   offsets of the first cell, stencil of the second:
 //                      make_layout's status (larger of the two cells' errors)
 #include <cuda_runtime.h>
@@ -14,7 +15,16 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "plan.h"
+static int g_scans = 0;   // questions whether a stencil's second-order operator is definite
+static bool counted_mg_definite(const exx::Stencil &st)
+{
+    ++g_scans;
+    return exx::mg_definite(st);
+}
+#define mg_definite counted_mg_definite
 #include "api.cu"
+#undef mg_definite
 
 static long long g_alloc = 0, g_fail_at = 0;
 static bool g_launched = false, g_match = false;
@@ -147,6 +157,9 @@ int main()
             int k;
             if (std::scanf("%d", &k) != 1) return 4;
             g_fail_at = k ? g_alloc + k : 0;
+        } else if (!std::strcmp(cmd, "scans")) {
+            std::printf("%d\n", g_scans);
+            g_scans = 0;
         } else if (!std::strcmp(cmd, "layout")) {
             exx_cell a{}, b{};
             double rpe, rme;

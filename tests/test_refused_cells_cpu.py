@@ -70,3 +70,15 @@ def test_failed_upload_is_made_again(harness, frozen, fail_at):
     r = run(harness, f"plan {PLAN} 48 48 48 4.0 {ROOMY} {frozen} 1 1", f"oom {fail_at}", f"step {SHEAR}", "oom 0",
             f"step {SHEAR}", f"step {SAME_DIRS}", f"step {PLAN}")
     assert r == [OK, [OOM, None], [OK, True], [OK, True], [OK, True]]
+
+
+@pytest.mark.parametrize("frozen", [1, 0])
+def test_definiteness_is_asked_when_the_stencil_changes(harness, frozen):
+    """A cell with a negative stencil coefficient: mg_definite scans 32^3 frequencies there."""
+    sheared, other = cell(1.1, 0.0, 0.0), cell(1.102, 0.0, 0.0)
+    r = run(harness, f"plan {sheared} 36 36 36 3.0 5.5 {frozen} 1 1", "scans", f"step {sheared}", f"step {sheared}", "scans",
+            f"step {other}", "scans", f"step {other}", "scans", f"plan {sheared} 36 36 36 3.0 5.5 {frozen} 1 0",
+            f"step {other}", "scans")
+    solved = [OK, True]
+    # once for a plan, not at all for its solves, once for another cell, never without the preconditioner
+    assert r == [OK, 1, solved, solved, 0, solved, 1, solved, 0, OK, solved, 0]
