@@ -2053,14 +2053,16 @@ __device__ __noinline__ void cg_fp64_mg(const SetDev &S, const SmemCell &sm, dou
     double pq_old = 0.0;
     for (;;) {
         // ended at a fifth of the bound: its error is then no larger than plain CG's, whose last
-        // iterations take smaller steps (one iteration more)
-        if (sqrt(rr) <= 0.2 * stop) {
+        // iterations take smaller steps (one iteration more).  A guess that meets the bound itself, and
+        // what the last allowed iteration leaves, count as they do for plain CG
+        const bool last = iters >= sm.C.max_iter;
+        if (sqrt(rr) <= (last || iters == 0 ? stop : 0.2 * stop)) {
             rr = residual_pass(S, vbox, rho, r64, sm.cw64, sm.ds, ndir, fdn, sm.center64, red);
             ++refine;
             if (sqrt(rr) <= stop) break;
             first = true;
         }
-        if (iters >= sm.C.max_iter || !(rr == rr)) {
+        if (last || !(rr == rr)) {
             status = 5;
             break;
         }
