@@ -179,12 +179,16 @@ def algorithmic_bytes(n_pairs, total_iter, total_refine, n_pe, n_me, s, mg_point
     the stencil, and the V-cycle's fine level: r read by each of its two
     stencil passes, z0 written and read, z written and read) plus 8 n_l s on
     every coarse level (its R, Z, T boxes written and read, Z read once more
-    by the prolongation, T by the restriction);
+    by the prolongation, T by the restriction); the FP64 path keeps 7 of these
+    accesses in FP64 and runs the V-cycle on an FP32 copy of r (written once more),
+    with FP32 coarse levels;
     true residual: FP64 path 24 N_PE (v, rho read, r written in FP64), mixed
     path 20 N_PE (v and 4 pi rho read as double-float pairs, r written in FP32);
     per pair: gather 2 N_ME 8, D read-modify-write 2 N_ME 16, rho 8 N_PE."""
     per_residual = 20.0 if s == 4 else 24.0
-    if mg_points:
+    if mg_points and s == 8:
+        per_iter = (7.0 * 8.0 + 7.0 * 4.0) * n_pe + 8.0 * 4.0 * sum(mg_points[1:])
+    elif mg_points:
         per_iter = 13.0 * n_pe * s + 8.0 * s * sum(mg_points[1:])
     else:
         per_iter = 7.0 * n_pe * s

@@ -207,10 +207,13 @@ typedef struct {
     int mg_points[6];
 } exx_plan_info;
 
-/* Schedule of a plan's mixed-precision pair solver (Step IV): the knobs that
- * change how fast the CG converges, never what it converges to (the stopping
- * rule |b - A v| <= cg_tol |b| on the true residual is fixed).  Set from
- * exx_params at plan creation; chosen per plan by exx_plan_autotune. */
+/* Schedule of a plan's pair solver (Step IV): the knobs that change how
+ * fast the CG converges, never what it converges to (the stopping rule
+ * |b - A v| <= cg_tol |b| on the true residual is fixed).  Set from exx_params at
+ * plan creation (EXX_PRECOND_NONE where there is no hierarchy); chosen per plan by
+ * exx_plan_autotune on the mixed path.  precond and omega are those that solves of
+ * either precision run with (plain CG in a cell that has no hierarchy);
+ * inner_shift concerns the mixed path alone. */
 typedef struct {
     int precond;            /* EXX_PRECOND_NONE or EXX_PRECOND_MG */
     float omega;            /* weighted-Jacobi factor of the V-cycle, in (0, 1] (default 0.8), as */
@@ -232,8 +235,8 @@ void exx_ctx_destroy(exx_ctx *ctx);
  * orbitals of extent box[].  It also sizes the context's workspace for the
  * plan -- the pair list (for all live plans of the context together, so that
  * they can be solved as one batch), the per-cell constants and the persistent
- * solver slots -- and, for the mixed path with EXX_PRECOND_MG, builds the
- * multigrid hierarchy on the host.  A solve with device-memory buffers then
+ * solver slots -- and, with EXX_PRECOND_MG, builds the multigrid hierarchy
+ * on the host.  A solve with device-memory buffers then
  * allocates nothing, with three exceptions: the first call with EXX_MEM_HOST
  * buffers allocates the plan's device staging copies; warm_start grows the
  * plan's solution stores when the pair count exceeds them; and a frozen-mode
@@ -286,7 +289,8 @@ int exx_pair_partition(const exx_cell *cell, const exx_params *params, int n_pai
 
 /* The plan's solver schedule (exx_schedule), and setting it by hand.
  * set: EXX_ERR_ARG for a value out of range, or EXX_PRECOND_MG on a plan
- * without a multigrid hierarchy (FP64 path, fd_order > 3, tiny subdomains). */
+ * without a multigrid hierarchy (created with EXX_PRECOND_NONE, fd_order > 3, tiny
+ * subdomains). */
 int exx_plan_get_schedule(const exx_plan *plan, exx_schedule *sched);
 int exx_plan_set_schedule(exx_plan *plan, const exx_schedule *sched);
 
@@ -298,8 +302,8 @@ int exx_plan_set_schedule(exx_plan *plan, const exx_schedule *sched);
  * timing the solver launch with CUDA events on `stream`, twice per candidate
  * (the faster run counts), and keeps the fastest for the plan's later solves
  * (ties keep the earlier candidate, the order above).  `chosen` (may be NULL)
- * receives it with its time.  The FP64 path has one schedule (of its parameters)
- * and returns it untimed.  A sample of several waves of the persistent grid
+ * receives it with its time.  The FP64 path keeps the schedule it has
+ * and returns it untimed (ms = 0).  A sample of several waves of the persistent grid
  * (a few times `ctas` of exx_plan_query) gives stable choices: with one wave
  * the slowest single pair decides each time.  cell and orb as for
  * exx_pairs_solve (device or host memory).  Errors: those of exx_pairs_solve,

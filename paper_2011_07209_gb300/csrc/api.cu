@@ -587,8 +587,7 @@ static void fill_celldev(const exx_plan *p, CellDev &C)
     C.r_pair2 = p->params.r_pair * p->params.r_pair;
     C.stress_mode = p->params.stress_mode;
     C.guess = p->params.guess;
-    // the FP64 path takes its preconditioner from the parameters: schedules are the mixed path's
-    C.precond = (p->params.precision == EXX_MIXED ? p->sched.precond : p->params.precond) && p->mg_ok;
+    C.precond = p->sched.precond && p->mg_ok;
     C.inner_shift = p->sched.inner_shift;
     C.mg_omega = (float)(p->sched.omega * mg_omega_scale(n));
     for (int s = 0; s < 2; ++s) {
@@ -860,9 +859,8 @@ int exx_plan_create(exx_ctx *ctx, const exx_cell *cell, const exx_params *params
     p->sched.omega = (float)kMgOmega;
     p->sched.inner_shift = ctx->inner_shift;
     e = build_geometry(p, *cell);
-    if (!e && p->sched.precond == EXX_PRECOND_MG &&
-        (params->precision != EXX_MIXED || (!p->d_mg[0] && !p->d_mg[1])))
-        p->sched.precond = EXX_PRECOND_NONE;   // no hierarchy for this plan (plain CG), or no schedule (FP64)
+    if (!e && p->sched.precond == EXX_PRECOND_MG && !p->d_mg[0] && !p->d_mg[1])
+        p->sched.precond = EXX_PRECOND_NONE;   // no hierarchy for this plan: plain CG
     if (!e) {
         const long long pairs = (long long)max_orb * (max_orb + 1) / 2;
         p->pairs_cap = (int)std::min<long long>(pairs, 1LL << 30);
@@ -1460,9 +1458,7 @@ int exx_plan_set_schedule(exx_plan *plan, const exx_schedule *sched)
     if (sched->precond != EXX_PRECOND_NONE && sched->precond != EXX_PRECOND_MG) return EXX_ERR_ARG;
     if (!(sched->omega > 0.f && sched->omega <= 1.f) || sched->inner_shift < 4 || sched->inner_shift > 22)
         return EXX_ERR_ARG;
-    if (sched->precond == EXX_PRECOND_MG &&
-        (plan->params.precision != EXX_MIXED || (!plan->d_mg[0] && !plan->d_mg[1])))
-        return EXX_ERR_ARG;
+    if (sched->precond == EXX_PRECOND_MG && !plan->d_mg[0] && !plan->d_mg[1]) return EXX_ERR_ARG;
     plan->sched = *sched;
     return EXX_OK;
 }
@@ -1474,7 +1470,6 @@ int exx_plan_autotune(exx_ctx *ctx, exx_plan *plan, const exx_cell *cell, const 
     std::vector<exx_schedule> cand =
         schedule_candidates(plan->params.precision == EXX_MIXED && (plan->d_mg[0] || plan->d_mg[1]), kMgOmega);
     if (plan->params.precision != EXX_MIXED) {
-        plan->sched.precond = EXX_PRECOND_NONE;
         plan->sched.ms = 0.0;
         if (chosen) *chosen = plan->sched;
         return EXX_OK;

@@ -7,6 +7,8 @@
 //                      layout that is the one of the stencil it was given
 //   oom <k>            the k-th device allocation from now on fails (0: none)
 //   scans              how often mg_definite was asked since the last time
+//   get | set <precond> <omega> | auto   exx_plan_get_schedule, _set_schedule, exx_plan_autotune
+//   seen               [V-cycle, its Jacobi weight] of the last launch
 //   layout <9 lattice> <3 n> <9 lattice> r_pe r_me   offsets of the first cell, stencil of the second:
 //                      make_layout's status (larger of the two cells' errors)
 #include <cuda_runtime.h>
@@ -28,6 +30,8 @@ static bool counted_mg_definite(const exx::Stencil &st)
 
 static long long g_alloc = 0, g_fail_at = 0;
 static bool g_launched = false, g_match = false;
+static int g_precond = 0;
+static float g_omega = 0.f;
 static exx_plan *g_plan = nullptr;
 static char g_event;
 
@@ -86,6 +90,8 @@ cudaError_t launch_solve(const CellDev *cells, const ListDev &, const SolveSlots
     // the layout that belongs to the directions that the kernels are given
     g_launched = g_match = true;
     const CellDev &C = cells[0];
+    g_precond = C.precond && C.set[1].mg;
+    g_omega = C.mg_omega;
     for (int s = 0; s < 2; ++s) {
         Stencil st = g_plan->stencil;
         for (int d = 0; d < C.ndir; ++d)
@@ -104,6 +110,11 @@ cudaError_t launch_solve(const CellDev *cells, const ListDev &, const SolveSlots
     return cudaSuccess;
 }
 }  // namespace exx
+
+static void show(int e, const exx_schedule &sc)
+{
+    std::printf("[%d, %d, %.4f, %d, %.1f]\n", e, sc.precond, sc.omega, sc.inner_shift, sc.ms);
+}
 
 static bool lattice(exx_cell &c)
 {
@@ -157,6 +168,22 @@ int main()
             int k;
             if (std::scanf("%d", &k) != 1) return 4;
             g_fail_at = k ? g_alloc + k : 0;
+        } else if (!std::strcmp(cmd, "get")) {
+            exx_schedule sc{};
+            const int e = exx_plan_get_schedule(g_plan, &sc);
+            show(e, sc);
+        } else if (!std::strcmp(cmd, "set")) {
+            exx_schedule sc{};
+            sc.inner_shift = 14;
+            if (std::scanf("%d %f", &sc.precond, &sc.omega) != 2) return 4;
+            std::printf("%d\n", exx_plan_set_schedule(g_plan, &sc));
+        } else if (!std::strcmp(cmd, "auto")) {   // (FP64 plans: nothing is launched)
+            exx_schedule sc{};
+            exx_orbitals o{};
+            const int e = exx_plan_autotune(ctx, g_plan, &c, &o, 1, &sc, nullptr);
+            show(e, sc);
+        } else if (!std::strcmp(cmd, "seen")) {
+            std::printf("[%d, %.4f]\n", g_precond, g_omega);
         } else if (!std::strcmp(cmd, "scans")) {
             std::printf("%d\n", g_scans);
             g_scans = 0;
