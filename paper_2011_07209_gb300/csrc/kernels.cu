@@ -2,7 +2,7 @@
 //
 //   k_tables       regular solid harmonics on PE points and far-field kernels
 //                  on shell points of one subdomain kind (Eqs. me, mepole)
-//   k_pair_rows    unique pair list, a few orbital rows per CTA (Step II)
+//   k_pair_rows    unique pair list, one to four orbital rows per CTA (Step II)
 //   k_pair_scan    row offsets and per-cell ranges of the pair list
 //   k_pair_solve   persistent: one CTA owns one pair at a time and runs the
 //                  whole per-pair path (Steps III-V): pair density, moments,
@@ -129,22 +129,21 @@ __global__ void k_tables(const CellDev *__restrict__ cell, int which, double *S6
 // ---------------------------------------------------------------------------
 // Pair list: the rule of pair_rule.cuh.
 // ---------------------------------------------------------------------------
-// kPairRows rows of one cell per CTA.  fill = 0: count; 1: write.
-__global__ void __launch_bounds__(kPairThreads) k_pair_rows(const CellDev *__restrict__ cells, int n_cells, ListDev L,
-                                                           int fill)
+// R rows of one cell per CTA.  Counts the rows' pairs, or writes them (FILL).
+template <int R, bool FILL>
+__global__ void __launch_bounds__(kPairThreads) k_pair_rows(const CellDev *__restrict__ cells, int n_cells, ListDev L)
 {
     int c = 0, b = blockIdx.x;
     for (; c < n_cells; ++c) {
-        const int nb = (cells[c].n_orb + kPairRows - 1) / kPairRows;
+        const int nb = (cells[c].n_orb + R - 1) / R;
         if (b < nb) break;
         b -= nb;
     }
     if (c == n_cells) return;
     const CellDev &C = cells[c];
-    const int i0 = b * kPairRows, row0 = C.row_base + i0;
-    int cnt[kPairRows];
-    pair_rows_block(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
-        if (!fill) return;
+    const int i0 = b * R, row0 = C.row_base + i0;
+    int cnt[R];
+    pair_rows_block<R, FILL>(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
         const int pos = L.row_start[row0 + r] + p;
         if (pos >= L.capacity) return;
         PairRec pr;
@@ -158,8 +157,8 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_rows(const CellDev *__res
         pr.pad = 0;
         L.pairs[pos] = pr;
     });
-    if (!fill && threadIdx.x == 0)
-        for (int r = 0; r < kPairRows && i0 + r < C.n_orb; ++r) L.row_count[row0 + r] = cnt[r];
+    if (!FILL && threadIdx.x == 0)
+        for (int r = 0; r < R && i0 + r < C.n_orb; ++r) L.row_count[row0 + r] = cnt[r];
 }
 
 // Exclusive scan of the row counts (single CTA), per-cell ranges, capacity check.
@@ -3830,12 +3829,20 @@ cudaError_t launch_guess_info(const int32_t *perm, const uint8_t *bin, const int
     return cudaGetLastError();
 }
 
+template <bool FILL>
+static void launch_pair_rows(const CellDev *cells, int n_cells, int n_rows, const ListDev &L, cudaStream_t s)
+{
+    const int R = pair_rows_per_cta(n_rows);
+    const int blocks = R > 1 ? n_rows / R + n_cells : n_rows;   // a cell's last rows may fill a CTA only in part
+    auto k = R == 1 ? k_pair_rows<1, FILL> : R == 2 ? k_pair_rows<2, FILL> : k_pair_rows<4, FILL>;
+    k<<<blocks, kPairThreads, 0, s>>>(cells, n_cells, L);
+}
+
 cudaError_t launch_pair_list(const CellDev *cells, int n_cells, int n_rows, const ListDev &L, cudaStream_t s)
 {
-    const int blocks = n_rows / kPairRows + n_cells;   // a cell's last rows may fill a CTA only in part
-    if (n_rows > 0) k_pair_rows<<<blocks, kPairThreads, 0, s>>>(cells, n_cells, L, 0);
+    if (n_rows > 0) launch_pair_rows<false>(cells, n_cells, n_rows, L, s);
     k_pair_scan<<<1, 1024, 0, s>>>(cells, n_cells, n_rows, L);
-    if (n_rows > 0) k_pair_rows<<<blocks, kPairThreads, 0, s>>>(cells, n_cells, L, 1);
+    if (n_rows > 0) launch_pair_rows<true>(cells, n_cells, n_rows, L, s);
     return cudaGetLastError();
 }
 

@@ -37,13 +37,13 @@ struct PairCell {
     int n_orb;
 };
 
-// kPairRows rows per CTA; fill = 0 counts, fill = 1 writes rows in (i, j) order.
-__global__ void __launch_bounds__(exx::kPairThreads) k_rows_noalloc(PairCell C, int *scratch, int fill, int cap, int *rows)
+// R rows per CTA: counts the rows' pairs, or writes them in (i, j) order (FILL).
+template <int R, bool FILL>
+__global__ void __launch_bounds__(exx::kPairThreads) k_rows_noalloc(PairCell C, int *scratch, int cap, int *rows)
 {
-    const int i0 = blockIdx.x * exx::kPairRows;
-    int cnt[exx::kPairRows];
-    exx::pair_rows_block(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
-        if (!fill) return;
+    const int i0 = blockIdx.x * R;
+    int cnt[R];
+    exx::pair_rows_block<R, FILL>(C, C.n_orb, i0, cnt, [&](int r, int p, int j, const int *kb, const int *g) {
         const int pos = scratch[kMaxOrbNoalloc + i0 + r] + p;
         if (pos >= cap) return;
         int *o = rows + 8 * (size_t)pos;
@@ -54,8 +54,16 @@ __global__ void __launch_bounds__(exx::kPairThreads) k_rows_noalloc(PairCell C, 
             o[5 + a] = g[a];
         }
     });
-    if (!fill && threadIdx.x == 0)
-        for (int r = 0; r < exx::kPairRows && i0 + r < C.n_orb; ++r) scratch[i0 + r] = cnt[r];
+    if (!FILL && threadIdx.x == 0)
+        for (int r = 0; r < R && i0 + r < C.n_orb; ++r) scratch[i0 + r] = cnt[r];
+}
+
+template <bool FILL>
+void launch_rows(const PairCell &C, int *scratch, int cap, int *rows, cudaStream_t s)
+{
+    const int R = exx::pair_rows_per_cta(C.n_orb);
+    auto k = R == 1 ? k_rows_noalloc<1, FILL> : R == 2 ? k_rows_noalloc<2, FILL> : k_rows_noalloc<4, FILL>;
+    k<<<(C.n_orb + R - 1) / R, exx::kPairThreads, 0, s>>>(C, scratch, cap, rows);
 }
 
 // Exclusive scan of the row counts (one CTA); writes the total to the scratch
@@ -180,10 +188,9 @@ extern "C" int exx_pair_list_noalloc(const exx_cell *cell, const double *centres
     C.n_orb = n_orb;
     cudaStream_t s = (cudaStream_t)stream;
     // the counts of every row are rewritten below; nothing else needs zeroing
-    const int blocks = (n_orb + exx::kPairRows - 1) / exx::kPairRows;
-    if (n_orb > 0) k_rows_noalloc<<<blocks, exx::kPairThreads, 0, s>>>(C, scratch, 0, cap, rows);
+    if (n_orb > 0) launch_rows<false>(C, scratch, cap, rows, s);
     k_scan_noalloc<<<1, 1024, 0, s>>>(scratch, n_orb, n_pairs);
-    if (n_orb > 0) k_rows_noalloc<<<blocks, exx::kPairThreads, 0, s>>>(C, scratch, 1, cap, rows);
+    if (n_orb > 0) launch_rows<true>(C, scratch, cap, rows, s);
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return exx::note_cuda_error("noalloc.cu: launch", ce);
     return EXX_OK;

@@ -9,7 +9,8 @@
 // g = NINT(N (s_i + (ds + k)/2)) mod N, NINT rounding half away from zero
 // (round()).  Every product and sum is an explicit round-to-nearest intrinsic,
 // so nothing is contracted and the operation order is the one the oracle uses.
-// The list of 1024 orbitals (count, scan, fill) on one GB300: 789 us with the rule on every pair, 98 us screened.
+// The list of 1024 orbitals (count, scan, fill) on one GB300, one pair in twenty near: 822 us with the rule on every
+// pair, 60 us screened; of 4 orbitals 37.6 -> 20.3, of 128 that are all near 41.6 -> 23.1, of 1024 that are 832 -> 222.
 #pragma once
 
 namespace exx {
@@ -35,21 +36,20 @@ __device__ __forceinline__ void pair_frac(const Cell &C, int i, double *s)
 // the screen cannot rule out, over the images that it cannot rule out.
 struct PairScreen {
     float h[3][3];
-    float H;   // largest sum of |h| over a row: a component's error per unit of coordinate error
     float r;   // R_pair
+    float H;   // largest sum of |h| over a row: a component's error per unit of coordinate error
+    // by the lanes of one warp, for the CTA (conversions from FP64 are slow): h and r
     template <class Cell>
-    __device__ explicit PairScreen(const Cell &C)
+    __device__ void fill(const Cell &C, int lane)
+    {
+        if (lane < 9) h[lane / 3][lane % 3] = (float)C.h[lane / 3][lane % 3];
+        if (lane == 9) r = sqrtf((float)C.r_pair2) * (1.f + 0x1p-20f);
+    }
+    __device__ void set_norm()
     {
         H = 0.f;
-        for (int a = 0; a < 3; ++a) {
-            float t = 0.f;
-            for (int b = 0; b < 3; ++b) {
-                h[a][b] = (float)C.h[a][b];
-                t += fabsf(h[a][b]);
-            }
-            H = fmaxf(H, t);
-        }
-        r = sqrtf((float)C.r_pair2) * (1.f + 0x1p-20f);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) H = fmaxf(H, fabsf(h[a][0]) + fabsf(h[a][1]) + fabsf(h[a][2]));
     }
     // error of a Cartesian component of h (ds + k) in FP32: es, that of ds, and the roundings of the
     // sums (|ds + k| < 2; 16 half-ulps cover them)
@@ -106,12 +106,11 @@ struct PairScreen {
     }
 };
 
-// The rule.
-template <class Cell>
-__device__ __forceinline__ bool pair_rule(const Cell &C, const PairScreen &scr, int i, int j, int *kb, int *g)
+// The rule.  si: the fractional coordinates of i; g is formed with GRID only.
+template <bool GRID, class Cell>
+__device__ __forceinline__ bool pair_rule(const Cell &C, const PairScreen &scr, const double *si, int j, int *kb, int *g)
 {
-    double si[3], ds[3];
-    pair_frac(C, i, si);
+    double ds[3];
     pair_frac(C, j, ds);
     for (int al = 0; al < 3; ++al) {
         const double d = __dadd_rn(ds[al], -si[al]);
@@ -135,6 +134,7 @@ __device__ __forceinline__ bool pair_rule(const Cell &C, const PairScreen &scr, 
         }
     }
     if (!(best <= C.r_pair2)) return false;
+    if (!GRID) return true;
     for (int al = 0; al < 3; ++al) {
         const double sm = __dadd_rn(si[al], __dmul_rn(__dadd_rn(ds[al], (double)kb[al]), 0.5));
         const long long gg = (long long)round(__dmul_rn((double)C.n[al], sm));
@@ -145,84 +145,138 @@ __device__ __forceinline__ bool pair_rule(const Cell &C, const PairScreen &scr, 
     return true;
 }
 
-// Rows i0 .. i0 + kPairRows - 1 of the list by one CTA of kPairThreads: screens every
-// j >= i of each row in FP32, collects the survivors in shared memory and runs the
-// rule on them with full warps.  emit(row, position, j, k, g) receives the pairs of a row in
-// ascending j, position counting from 0; returns the rows' pair counts in cnt (every thread).
-constexpr int kPairRows = 4, kPairThreads = 256, kPairList = 1024;
-template <class Cell, class Emit>
-__device__ void pair_rows_block(const Cell &C, int n_orb, int i0, int *cnt, Emit emit)
+// Rows i0 .. i0 + R - 1 of the list by one CTA of kPairThreads: screens every j >= i of each
+// row in FP32, collects the survivors in shared memory (a list per row) and runs the rule on the
+// lists of all rows together, a warp on 32 survivors of one row, so that no warp of the CTA
+// waits while another row's survivors are ruled.  What every thread needs in FP64 of the
+// rows and the cell is formed once per CTA.  emit(r, position, j, k, g) receives the pairs of row
+// i0 + r in ascending j, position counting from 0 (FILL only); cnt: the rows' pair counts (every thread).
+constexpr int kPairThreads = 256, kPairWarps = kPairThreads / 32, kPairList = 1024;
+template <int R, bool FILL, class Cell, class Emit>
+__device__ __forceinline__ void pair_rows_block(const Cell &C, int n_orb, int i0, int (&cnt)[R], Emit emit)
 {
-    __shared__ int s_list[kPairRows][kPairList];
-    __shared__ int s_warp[kPairRows][kPairThreads / 32];
+    __shared__ PairScreen s_scr;
+    __shared__ double s_si[R][3];
+    __shared__ float s_sif[R][3];
+    __shared__ int s_list[R][kPairList];
+    __shared__ int s_warp[2][R][kPairWarps];   // two buffers: one barrier per step
+    __shared__ int s_run[2][kPairWarps];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const PairScreen scr(C);
-    float si[kPairRows][3];
-#pragma unroll
-    for (int r = 0; r < kPairRows; ++r) {
-        double s[3] = {0.0, 0.0, 0.0};
-        if (i0 + r < n_orb) pair_frac(C, i0 + r, s);
-        for (int al = 0; al < 3; ++al) si[r][al] = (float)s[al];
-        cnt[r] = 0;
+    const unsigned below = (1u << lane) - 1u;
+    if (w == 0 && lane < 3 * R) {
+        const int r = lane / 3, al = lane - 3 * r;
+        double s = 0.0;
+        if (i0 + r < n_orb) {
+            const double *c = C.centres + 3 * (i0 + r);
+            s = pair_dot3_rn(C.hinv[al], c[0], c[1], c[2]);
+        }
+        s_si[r][al] = s;
+        s_sif[r][al] = (float)s;
     }
-    int len[kPairRows] = {};
-    // sum over the CTA's warps of a per-warp count, and the part of the warps before this one
-    auto scan = [&](int r, int mine, int &before, int &total) {
-        if (lane == 0) s_warp[r][w] = mine;
-        __syncthreads();
-        before = total = 0;
-        for (int k = 0; k < kPairThreads / 32; ++k) {
-            if (k < w) before += s_warp[r][k];
-            total += s_warp[r][k];
-        }
-    };
-    auto flush = [&](int r) {   // the rule on the row's survivors, in order
-        __syncthreads();
-        for (int p0 = 0; p0 < len[r]; p0 += kPairThreads) {
-            int kb[3], g[3];
-            const int j = p0 + tid < len[r] ? s_list[r][p0 + tid] : -1;
-            const bool ok = j >= 0 && pair_rule(C, scr, i0 + r, j, kb, g);
-            const unsigned bal = __ballot_sync(0xffffffffu, ok);
-            int before, total;
-            scan(r, __popc(bal), before, total);
-            if (ok) emit(r, cnt[r] + before + __popc(bal & ((1u << lane) - 1u)), j, kb, g);
-            cnt[r] += total;
-            __syncthreads();
-        }
-        len[r] = 0;
-    };
-    for (int j0 = i0; j0 < n_orb; j0 += kPairThreads) {
-        const int j = j0 + tid;
-        float sj[3] = {0.f, 0.f, 0.f};
-        if (j < n_orb) {
-            double s[3];
-            pair_frac(C, j, s);
-            for (int al = 0; al < 3; ++al) sj[al] = (float)s[al];
-        }
-        unsigned bal[kPairRows];
+    if (w == 1) s_scr.fill(C, lane);
+    __syncthreads();
+    PairScreen scr = s_scr;
+    scr.set_norm();
+    int len[R];
 #pragma unroll
-        for (int r = 0; r < kPairRows; ++r) {
-            bal[r] = __ballot_sync(0xffffffffu, j < n_orb && j >= i0 + r && i0 + r < n_orb && scr.near(si[r], sj));
-            if (lane == 0) s_warp[r][w] = __popc(bal[r]);
-        }
-        __syncthreads();
+    for (int r = 0; r < R; ++r) cnt[r] = len[r] = 0;
+    auto pick = [](const int (&v)[R], int r) {   // v[r] from registers
+        int x = 0;
 #pragma unroll
-        for (int r = 0; r < kPairRows; ++r) {
-            int before = len[r], total = 0;
-            for (int k = 0; k < kPairThreads / 32; ++k) {
-                if (k < w) before += s_warp[r][k];
-                total += s_warp[r][k];
+        for (int k = 0; k < R; ++k) x = k == r ? v[k] : x;
+        return x;
+    };
+    auto flush = [&]() {   // the rule on the survivors of every row, in order
+        __syncthreads();
+        int nw = 0;   // warps' worth of survivors
+#pragma unroll
+        for (int r = 0; r < R; ++r) nw += (len[r] + 31) >> 5;
+        for (int q0 = 0, buf = 0; q0 < nw; q0 += kPairWarps, buf ^= 1) {
+            int r = 0, b = q0 + w;   // this warp's row, and its place in the row's list
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int n = (len[k] + 31) >> 5;
+                if (r == k && b >= n) {
+                    b -= n;
+                    ++r;
+                }
             }
-            if (bal[r] >> lane & 1u) s_list[r][before + __popc(bal[r] & ((1u << lane) - 1u))] = j;
-            len[r] += total;
+            const int p = (b << 5) + lane;
+            int kb[3], g[3], j = -1;
+            bool ok = false;
+            if (r < R && p < pick(len, r)) {
+                j = s_list[r][p];
+                ok = pair_rule<FILL>(C, scr, s_si[r], j, kb, g);
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, ok);
+            if (lane == 0) s_run[buf][w] = r << 8 | __popc(bal);
+            __syncthreads();
+            if constexpr (FILL) {
+                int pos = r < R ? pick(cnt, r) + __popc(bal & below) : 0;
+#pragma unroll
+                for (int k = 0; k < kPairWarps; ++k)
+                    if (k < w && s_run[buf][k] >> 8 == r) pos += s_run[buf][k] & 255;
+                if (ok) emit(r, pos, j, kb, g);
+            }
+#pragma unroll
+            for (int k = 0; k < kPairWarps; ++k) {
+                const int rk = s_run[buf][k] >> 8, n = s_run[buf][k] & 255;
+#pragma unroll
+                for (int x = 0; x < R; ++x) cnt[x] += rk == x ? n : 0;
+            }
         }
+#pragma unroll
+        for (int r = 0; r < R; ++r) len[r] = 0;
         __syncthreads();
+    };
+    for (int j0 = i0, buf = 0; j0 < n_orb; j0 += kPairThreads, buf ^= 1) {
+        const int j = j0 + tid;
+        unsigned bal[R];
 #pragma unroll
-        for (int r = 0; r < kPairRows; ++r)
-            if (len[r] > kPairList - kPairThreads) flush(r);
+        for (int r = 0; r < R; ++r) bal[r] = 0;
+        if (j0 + 32 * w < n_orb) {   // (the whole warp; FP64 below)
+            float sj[3] = {0.f, 0.f, 0.f};
+            if (j < n_orb) {
+                double s[3];
+                pair_frac(C, j, s);
+                for (int al = 0; al < 3; ++al) sj[al] = (float)s[al];
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                bal[r] = __ballot_sync(0xffffffffu, j < n_orb && j >= i0 + r && i0 + r < n_orb && scr.near(s_sif[r], sj));
+        }
+        if (lane == 0)
+#pragma unroll
+            for (int r = 0; r < R; ++r) s_warp[buf][r][w] = __popc(bal[r]);
+        __syncthreads();
+        bool full = false;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            int before = len[r], total = 0;
+#pragma unroll
+            for (int k = 0; k < kPairWarps; ++k) {
+                if (k < w) before += s_warp[buf][r][k];
+                total += s_warp[buf][r][k];
+            }
+            if (bal[r] >> lane & 1u) s_list[r][before + __popc(bal[r] & below)] = j;
+            len[r] += total;
+            full |= len[r] > kPairList - kPairThreads;
+        }
+        if (full) flush();
     }
-#pragma unroll
-    for (int r = 0; r < kPairRows; ++r) flush(r);
+    flush();
 }
+
+// Rows per CTA (R) for a list of n rows: the rows of a CTA share the FP64 coordinates of the columns,
+// which bound the screen, but their survivors share its warps and the grid shrinks.  Measured, one
+// GB300, the whole list of n orbitals in us with R = 1 / 2 / 4, one pair in twenty near, and all:
+//    n =  256   23.6 /  23.2 /  27.2    36.0 /  43.6 /  68.4
+//    n =  512   39.5 /  31.3 /  35.4    83.1 /  86.5 / 125
+//    n = 1024   76.4 /  60.3 /  59.9     208 /   222 /  292
+//    n = 1500    132 /  98.8 /  90.7     410 /   410 /  507
+//    n = 2048    221 /   154 /   132     734 /   698 /  754
+//    n = 4096    762 /   505 /   384    2830 /  2620 /  2550
+// Two rows once they leave each of the 152 SMs a CTA, four once that leaves two.
+inline int pair_rows_per_cta(int n) { return n < 2 * 152 ? 1 : n < 8 * 152 ? 2 : 4; }
 
 }  // namespace exx
