@@ -9,7 +9,7 @@ re-sampled; frozen proto-subdomains (offsets of step 0, Sec. III B 2),
 R_pair / R_PE / R_ME = 8 / 6 / 8 bohr, 37-point NK stencil, CG tol 1e-9.  One
 bench step = one full EXX evaluation of the next MD step (pair list -> every
 pair's Poisson solve -> E_xx, D_xx, sigma_xx / Pi_xx) with the orbitals
-resident in HBM, the mixed FP32/FP64 path.  The same line carries the plain
+resident in HBM, the mixed FP32/FP64 path.  The same line carries the
 FP64 GPU path on a pair sample of MD step 0 (with the mixed path on the same
 sample), both paths' errors against the FP64 oracle on that sample, the
 end-to-end rate through the C ABI with host buffers, and the oracle's own rate

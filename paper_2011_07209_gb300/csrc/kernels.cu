@@ -1539,11 +1539,12 @@ __device__ __noinline__ void mg_coarse_cycle()
     const int tid = threadIdx.x, nt = blockDim.x;
     const int L = m.nlev - 1;   // coarsest
     // down: Jacobi smoothing from zero, Z = D R, its residual T = R - A Z, restriction.
-    // Level 1 (the largest coarse level, 8x fewer points than the fine one but 81-99
+    // Level 1 (the largest coarse level: 8x fewer points than the fine one, but up to 27
     // pattern entries per row) skips the pre-smoothing: R_1 itself is restricted and
     // Z_1 starts from the coarse correction.  The cycle is then not exactly
     // symmetric; CG still takes it as a preconditioner (one iteration more at most on
-    // the benchmark cells, against one residual pass of level 1 less per cycle).
+    // the benchmark cells, against one residual pass of level 1 less per cycle; both
+    // measured with the sixth-order cycle, whose rows held 81 to 99 entries).
     for (int l = 1; l < L; ++l) {
         const int *pts = m.pts[l];
         const float *R = m.R[l];
@@ -1895,9 +1896,7 @@ __device__ __noinline__ void cg_mixed_mg(const CgMixed &cg, float *zf, float *mg
     float2 *vb = reinterpret_cast<float2 *>(cg.vbox);
     float *r32 = reinterpret_cast<float *>(cg.r64);
     const int32_t *__restrict__ poff = S.pe_off;
-    const int32_t *__restrict__ grp = S.groups;
-    const int npe = S.n_pe, ng = S.n_groups, ndir = cg.ndir;
-    const int *rs = S.rstride, *dsf = S.dstride;
+    const int npe = S.n_pe, ndir = cg.ndir;
     const double stop = cg.stop, inner_red = cg.inner_red;
     float2 *red2 = reinterpret_cast<float2 *>(cg.red);
     const int B1 = S.B[1], B2 = S.B[2];

@@ -134,13 +134,14 @@ __device__ __forceinline__ bool pair_rule(const Cell &C, const PairScreen &scr, 
         }
     }
     if (!(best <= C.r_pair2)) return false;
-    if (!GRID) return true;
-    for (int al = 0; al < 3; ++al) {
-        const double sm = __dadd_rn(si[al], __dmul_rn(__dadd_rn(ds[al], (double)kb[al]), 0.5));
-        const long long gg = (long long)round(__dmul_rn((double)C.n[al], sm));
-        long long r = gg % C.n[al];
-        if (r < 0) r += C.n[al];
-        g[al] = (int)r;
+    if constexpr (GRID) {
+        for (int al = 0; al < 3; ++al) {
+            const double sm = __dadd_rn(si[al], __dmul_rn(__dadd_rn(ds[al], (double)kb[al]), 0.5));
+            const long long gg = (long long)round(__dmul_rn((double)C.n[al], sm));
+            long long r = gg % C.n[al];
+            if (r < 0) r += C.n[al];
+            g[al] = (int)r;
+        }
     }
     return true;
 }
