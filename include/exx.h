@@ -251,7 +251,8 @@ int exx_plan_query(const exx_plan *plan, exx_plan_info *info);
 /* Evaluate E_xx, D_xx and sigma_xx / Pi_xx for one cell (Steps II-V).
  * `cell` may differ from the plan's cell: with params.frozen = 1 the plan's
  * offsets and aux directions are kept and every metric quantity follows the
- * new cell (Sec. III B 2); otherwise the plan is rebuilt for it.  On
+ * new cell (Sec. III B 2); otherwise the plan is rebuilt for it.  A cell that is
+ * refused (EXX_ERR_CELL, _NK, _HALO, _ARG) leaves the plan as it was.  On
  * EXX_ERR_CG_NOT_CONVERGED the other outputs are still written. */
 int exx_pairs_solve(exx_ctx *ctx, exx_plan *plan, const exx_cell *cell, const exx_orbitals *orb,
                     exx_result *res, void *stream);
